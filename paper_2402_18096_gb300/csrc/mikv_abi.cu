@@ -413,22 +413,19 @@ mikv_status mikv_prefill_scores(const mikv_shape* shape, const void* q_pre, cons
   if (!make_map(&a.map_q, q_pre, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, kHeadDim, qrows, 2 * kHeadDim, 64, kPfTile,
                 CU_TENSOR_MAP_SWIZZLE_128B) ||
       !make_map(&a.map_k, k_pre, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, kHeadDim, krows, 2 * kHeadDim, 64, kPfTile,
-                CU_TENSOR_MAP_SWIZZLE_128B) ||
-      !make_map(&a.map_q_str, q_pre, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, kHeadDim, qrows, 2 * kHeadDim, 64, kPfTile / 2,
-                CU_TENSOR_MAP_SWIZZLE_128B) ||
-      !make_map(&a.map_k_str, k_pre, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, kHeadDim, krows, 2 * kHeadDim, 64, kPfTile / 2,
                 CU_TENSOR_MAP_SWIZZLE_128B))
     return MIKV_ERR_CUDA;
   char* wsb = static_cast<char*>(workspace);
   a.status = reinterpret_cast<int*>(wsb);
   a.stats = reinterpret_cast<float*>(wsb + kWsHeader);
   a.scores = scores;
+  a.batch = shape->batch;
   a.heads_q = shape->heads_q;
   a.heads_kv = shape->heads_kv;
   a.T = T;
   a.T_pad = prefill_padded(T);
   a.scale_log2 = sm_scale * 1.4426950408889634f;
-  return cuda_status(launch_prefill(a, shape->batch, static_cast<cudaStream_t>(stream)));
+  return cuda_status(launch_prefill(a, static_cast<cudaStream_t>(stream)));
 }
 
 mikv_status mikv_decode_attention(const mikv_shape* shape, const mikv_cache* cache, int32_t n_lo, const void* q,

@@ -1186,10 +1186,6 @@ __device__ __forceinline__ void insert_row(const AttnArgs& a, int bh, int slot, 
   __syncwarp();
 }
 
-__device__ __forceinline__ void fence_proxy_async() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
 template <int BITS, int GROUP, int HB, int G, bool KCH = false>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm) attention_kernel(const __grid_constant__ AttnArgs a) {
   constexpr LoUnit U = KCH ? lo_unit_layout_kch(BITS, GROUP) : lo_unit_layout(BITS, GROUP);
@@ -1409,7 +1405,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) attention_kernel(const _
     cursor_next(cc, hu, n_u);
     __syncwarp();
     if (lane == 0 && u + kNS < u1) {
-      fence_proxy_async();  // our generic reads of this stage precede the next asynchronous write
+      fence_proxy_async_smem();  // our generic reads of this stage precede the next asynchronous write
       issue_unit<BITS, GROUP, HB, KCH>(a, ci, stage, bars + 8 * s, pol);
       cursor_next(ci, hu, n_u);
     }

@@ -4,18 +4,40 @@
 // arxiv 2402.18096).
 //
 // Two passes over the causal score matrix S = sm_scale * Q K^T, each a tiled bf16 contraction on the
-// fifth-generation tensor cores (tcgen05.mma, M = 128, N = 64, fp32 accumulators in tensor memory) fed by TMA:
+// fifth-generation tensor cores (tcgen05.mma, M = N = 128, fp32 accumulators in tensor memory) fed by TMA:
 //   1. rows:    per query i, the log2 of its softmax normaliser, c_i = log2 sum_{t <= i} 2^(s_it log2 e)
 //               (accumulated online against a reference, as in flash attention, without values);
 //   2. columns: per key t, sum over the G query heads and the queries i >= t of 2^(s_it log2 e - c_i).
-// A CTA owns one 128-token tile of its fixed operand (queries in pass 1, keys in pass 2: the M side, so that
-// epilogue thread r owns accumulator row r = TMEM lane r) and streams 64-token tiles of the other operand.
-// Its warps specialise: warp 8 issues the TMA copies (the fixed tile, then a four-stage ring of 128B-swizzled
-// streamed tiles, with pass 2's query normalisers), warp 9 issues the eight K = 16 MMAs of each tile into one
-// of four TMEM accumulators, and warps 0-7 (two per accumulator lane quarter, one per column half) read
-// their accumulator rows with tcgen05.ld, release them, and do the softmax arithmetic (an exponential per
-// score). The roles hand tiles over through mbarriers only; every wait is bounded in time and gives up when
-// another role has failed. Only the causal triangle is visited.
+// A work item is MT 128-token tiles of the fixed operand (queries in pass 1, keys in pass 2: the M side, so that an
+// epilogue thread owns one accumulator row = TMEM lane) and every 128-token tile of the other operand it meets in the
+// causal triangle.
+//
+// What bounds it: one exponential per score and pass (32 per clock and SM: 512 clocks per 128 x 128 tile) weighs as
+// much as the tile's MMAs (512 clocks at the tensor peak), so both have to run all the time.
+//  - Two warps issue MMAs, one per fixed tile. The issuing thread is held while its MMAs run and then spends about
+//    450 clocks on the hand-over (measured: 0, 4, 8 and 16 MMAs a tile took 446, 726, 993 and 1466 clocks), so one
+//    thread alone leaves the tensor cores idle half of the time; the other's MMAs fill its gap.
+//  - Two accumulators per fixed tile, so that MMAs run under the arithmetic, and one streamed tile for two fixed ones
+//    (MT = 2), which halves the traffic from L2 per score (the 128-row tiles drew 7.9 TB/s).
+//  - Four sets of four epilogue warps, one set per accumulator, each warp taking whole rows of 128 columns: a hand-over
+//    costs the same whatever the columns behind it. Four warps per scheduler hide each other's tcgen05.ld and
+//    barriers (158 clocks per 32 columns of a warp against 195 with two, 135 for the exponentials alone), so nothing
+//    is prefetched, which keeps the threads within the 96 registers of 19 warps, and one copy of the arithmetic
+//    keeps the loop in the instruction cache.
+//  - One persistent CTA per SM whose copies and MMAs run on into the next item (with one item per CTA, filling and
+//    draining cost 9 % of the 4096-token prefill). Items are handed out by the hardware's launch control (a running
+//    CTA takes over the block index of one that has not started), so long and short items balance without a counter
+//    in memory.
+//
+// Where the time goes now (128 x 128 tile and pass, clocks per SM): 1010 of the 512 that exponentials and MMAs each
+// need; MMAs with no arithmetic behind them 770, the arithmetic with no MMAs 790 (pass 1) and 930 (pass 2, whose
+// normalisers come from shared memory). B 8, H 32, T 4096: 1211 -> 1022 us; B 1, Hq 32 / Hkv 8, T 32768: 8.59 -> 7.27
+// ms against one CTA per 128-token tile with 64-token streamed tiles, two per SM.
+//
+// The CTA's warps specialise: warps 0 .. 8 MT - 1 take the accumulator rows with tcgen05.ld and do the softmax
+// arithmetic; one warp fetches the next item and issues the TMA copies (fixed tiles and a ring of 128B-swizzled
+// streamed tiles, with pass 2's query normalisers), two issue the MMAs. The roles hand tiles over through mbarriers
+// only; every wait is bounded in time and gives up when another role has failed.
 #include <math.h>
 
 #include "mikv_device.cuh"
@@ -25,185 +47,368 @@
 namespace mikv {
 namespace {
 
-constexpr int kPfN = 64;                                // tokens of a streamed tile (the MMA's N)
-constexpr int kPfEpiWarps = 8;                          // two per accumulator lane quarter: one per column half
-constexpr int kPfCols = kPfN / 2;                       // accumulator columns of one epilogue thread
-constexpr int kPfThreads = 32 * (kPfEpiWarps + 2);      // warps 0-7 epilogue, 8 copies, 9 MMAs
-constexpr int kPfCopyWarp = kPfEpiWarps, kPfMmaWarp = kPfEpiWarps + 1;
-constexpr int kPfFixBytes = kPfTile * kHeadDim * 2;     // 32 KB: the fixed 128 x 128 bf16 tile
-constexpr int kPfFixHalf = kPfTile * 128;               // one 64-channel box of it
-constexpr int kPfStrBytes = kPfN * kHeadDim * 2;        // 16 KB: a streamed 64 x 128 tile
-constexpr int kPfStrHalf = kPfN * 128;
-constexpr int kPfStages = 4;                            // streamed tiles in flight
-constexpr int kPfAcc = 4;                               // TMEM accumulators of kPfN columns
-constexpr int kPfTmemCols = kPfAcc * kPfN;
-constexpr int kPfStatBytes = kPfN * 4;                 // pass 2: the streamed queries' log2 normalisers
-constexpr int kPfBars = 1 + 5 * kPfStages + 1;          // fixed, full/free/acc-full/acc-empty/stats x 4, drain
-constexpr int kPfSmem = kPfFixBytes + kPfStages * (kPfStrBytes + kPfStatBytes) + 8 * kPfBars + 1024;
-static_assert(kPfTile == 128 && kPfStages == kPfAcc, "one accumulator row per epilogue thread; shared indices");
+constexpr int kPfTileBytes = kPfTile * kHeadDim * 2;    // 32 KB: 128 tokens x 128 channels, two 64-channel boxes
+constexpr int kPfHalf = kPfTile * 128;                  // one of the boxes
+constexpr int kPfCols = 32;                             // accumulator columns of one tcgen05.ld
+constexpr int kPfStages = 3;                            // streamed tiles in flight
+constexpr int kPfFix = 3;                               // fixed tiles: the current ones and the next item's first
+constexpr int kPfStatBytes = kPfTile * 4;               // pass 2: the streamed queries' log2 normalisers
+constexpr int kPfBars = 3 * kPfStages + 2 * kPfFix + 8 + 4 + 4 + 1;
+constexpr int kPfSmem =
+    1024 + (kPfFix + kPfStages) * kPfTileBytes + kPfStages * kPfStatBytes + 2 * 16 + 8 * kPfBars;
+static_assert(kPfSmem <= 227 * 1024, "shared memory of one SM");
+constexpr int kPfTmemCols = 512;                        // two accumulators of 128 columns per fixed tile
+__host__ __device__ constexpr int pf_threads(int MT) { return 32 * (8 * MT + 3); }  // epilogue, copies, 2 x MMA
 
 struct PfSmem {
-  uint32_t fixed, stage0, stat0, bars;
-  const uint8_t* gbase;  // generic address of `fixed`
-  __device__ uint32_t stage(int s) const { return stage0 + s * kPfStrBytes; }
-  __device__ uint32_t stat(int s) const { return stat0 + s * kPfStatBytes; }
-  __device__ const float* stat_ptr(int s) const { return reinterpret_cast<const float*>(gbase + (stat(s) - fixed)); }
-  __device__ uint32_t bar_fixed() const { return bars; }
-  __device__ uint32_t full(int s) const { return bars + 8 * (1 + s); }                 // copy landed
-  __device__ uint32_t sfree(int s) const { return bars + 8 * (1 + kPfStages + s); }    // MMAs read it
-  __device__ uint32_t tfull(int d) const { return bars + 8 * (1 + 2 * kPfStages + d); }  // accumulator ready
-  __device__ uint32_t tempty(int d) const { return bars + 8 * (1 + 3 * kPfStages + d); } // accumulator read
-  __device__ uint32_t sdone(int s) const { return bars + 8 * (1 + 4 * kPfStages + s); }   // stats read
-  __device__ uint32_t drain() const { return bars + 8 * (1 + 5 * kPfStages); }
+  uint32_t base;
+  __device__ uint32_t fixed(int f) const { return base + f * kPfTileBytes; }
+  __device__ uint32_t stage(int s) const { return base + (kPfFix + s) * kPfTileBytes; }
+  __device__ uint32_t stat(int s) const { return stage(kPfStages) + s * kPfStatBytes; }
+  __device__ uint32_t item(int k) const { return stat(kPfStages) + 16 * k; }
+  __device__ uint32_t bar(int i) const { return item(2) + 8 * i; }
+  __device__ uint32_t full(int s) const { return bar(s); }                      // copy landed
+  __device__ uint32_t sfree(int s) const { return bar(kPfStages + s); }         // MMAs read it
+  __device__ uint32_t sdone(int s) const { return bar(2 * kPfStages + s); }     // normalisers read
+  __device__ uint32_t ffull(int f) const { return bar(3 * kPfStages + f); }     // fixed tile landed
+  __device__ uint32_t ffree(int f) const { return bar(3 * kPfStages + kPfFix + f); }
+  __device__ uint32_t tfull(int d) const { return bar(3 * kPfStages + 2 * kPfFix + d); }  // accumulator ready
+  __device__ uint32_t tempty(int d) const { return bar(3 * kPfStages + 2 * kPfFix + 4 + d); }  // and read
+  __device__ uint32_t ifull(int k) const { return bar(3 * kPfStages + 2 * kPfFix + 8 + k); }   // next item known
+  __device__ uint32_t iempty(int k) const { return bar(3 * kPfStages + 2 * kPfFix + 10 + k); }
+  __device__ uint32_t pfull(int m) const { return bar(3 * kPfStages + 2 * kPfFix + 12 + m); }  // row partials there
+  __device__ uint32_t pempty(int m) const { return bar(3 * kPfStages + 2 * kPfFix + 14 + m); }  // and taken
+  __device__ uint32_t drain() const { return bar(kPfBars - 1); }
 };
 
-__device__ __forceinline__ PfSmem pf_smem() {
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  PfSmem r;
-  r.fixed = base;
-  r.gbase = smem_raw + (base - smem_u32(smem_raw));
-  r.stage0 = base + kPfFixBytes;
-  r.stat0 = r.stage0 + kPfStages * kPfStrBytes;
-  r.bars = r.stat0 + kPfStages * kPfStatBytes;
-  return r;
-}
-
-// Bounded wait that also gives up as soon as another role of the CTA has failed.
+// Bounded wait that also gives up as soon as another role of the CTA has failed. The clock is read only every 64
+// polls: a first read before the polls delays every wait that is not already over.
 __device__ __forceinline__ bool pf_wait(uint32_t bar, uint32_t parity, volatile int* fail) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = global_timer_ns();
+  uint64_t t0 = 0;
   for (uint32_t i = 1;; ++i) {
     if (mbar_try_wait(bar, parity)) return true;
-    if ((i & 63u) == 0 && (*fail || global_timer_ns() - t0 > kWaitLimitNs)) {
-      *fail = 1;
-      return false;
+    if ((i & 63u) == 0) {
+      const uint64_t t = global_timer_ns();
+      if (t0 == 0) t0 = t;
+      if (*fail || t - t0 > kWaitLimitNs) {
+        *fail = 1;
+        return false;
+      }
     }
   }
 }
 
-// The eight K = 16 MMAs of one tile: D (128 x 64) = fixed tile x streamed tile^T over the 128 channels.
+// The eight K = 16 MMAs of one tile: D (128 x 128) = fixed tile x streamed tile^T over the 128 channels.
 __device__ __forceinline__ void pf_mma_tile(uint32_t d_tmem, uint32_t fix, uint32_t str) {
-  constexpr uint32_t idesc = umma_idesc_bf16_f32(kPfTile, kPfN);
+  constexpr uint32_t idesc = umma_idesc_bf16_f32(kPfTile, kPfTile);
 #pragma unroll
   for (int ks = 0; ks < 8; ++ks) {
-    const uint32_t k = (ks & 3) * 32;  // channels 16 ks .. 16 ks + 15 inside their 64-channel box
-    umma_bf16(d_tmem, umma_desc_sw128(fix + (ks >> 2) * kPfFixHalf + k),
-              umma_desc_sw128(str + (ks >> 2) * kPfStrHalf + k), idesc, ks > 0 ? 1u : 0u);
+    const uint32_t k = (ks >> 2) * kPfHalf + (ks & 3) * 32;  // channels 16 ks .. + 15 inside their 64-channel box
+    umma_bf16(d_tmem, umma_desc_sw128(fix + k), umma_desc_sw128(str + k), idesc, ks > 0 ? 1u : 0u);
   }
 }
 
-// The pipeline shared by both passes: warp 8 streams the n_tiles tiles (rows str_row(n) of map_str) behind
-// the fixed tile (rows fix_row .. + 127 of map_fix), warp 9 multiplies each into one of four TMEM
-// accumulators, and warps 0-7 hand accumulator row halves to epi(n, col0, v): warp w gets row 32 (w % 4) +
-// lane, columns col0 = 32 (w / 4) .. col0 + 31. Returns false when a wait timed out (after draining what was
-// in flight); every role leaves through the final barrier.
-// STATS (pass 2): the copy warp also stages each streamed tile's kPfN query normalisers (stats + stat_off(n),
-// 16-byte aligned in the padded rows) with the tile; the epilogue warps release them through sdone.
-template <bool STATS, class StrRow, class StatOff, class Epi>
-__device__ __forceinline__ bool pf_pipeline(const PrefillArgs& a, const CUtensorMap* map_fix, int fix_row,
-                                            const CUtensorMap* map_str, int n_tiles, StrRow str_row,
-                                            StatOff stat_off, Epi epi) {
+// The work of block index lin. Heads are taken in groups (group_rows / group_cols of them), whole groups one after
+// another: inside a group all heads' longest items come first (so the last items of the grid are short ones), and
+// the group's streamed operand (of the heads that run at the same time) stays within L2.
+// PASS 1: queries q0 .. of query head `head` (b Hq + j), streamed keys 0 .. of its KV head.
+// PASS 2: keys q0 .. of KV head `head`, streamed queries q0 .. of its G query heads.
+template <int MT, int PASS>
+struct PfWork {
+  int head, q0, heads, n_tiles, str_row, stat_row, m_used;
+
+  __device__ __forceinline__ PfWork(const PrefillArgs& a, int lin) {
+    const int G = a.heads_q / a.heads_kv, n_heads = a.batch * (PASS == 1 ? a.heads_q : a.heads_kv);
+    const int items = (a.T + MT * kPfTile - 1) / (MT * kPfTile), per = PASS == 1 ? a.group_rows : a.group_cols;
+    const int grp = lin / (per * items), rem = lin - grp * per * items;
+    const int n = min(per, n_heads - grp * per);  // heads of this group
+    const int it = rem / n;
+    head = grp * per + (rem - it * n);
+    q0 = MT * kPfTile * (PASS == 1 ? items - 1 - it : it);
+    m_used = a.T - q0 > kPfTile ? MT : 1;  // fixed tiles that hold a token
+    if (PASS == 1) {
+      heads = 1;
+      n_tiles = (min(q0 + MT * kPfTile, a.T) + kPfTile - 1) / kPfTile;
+      str_row = head / G * a.T;
+      stat_row = 0;
+    } else {
+      heads = G;
+      n_tiles = (a.T - q0 + kPfTile - 1) / kPfTile;
+      str_row = head * G * a.T + q0;
+      stat_row = head * G * a.T_pad + q0;
+    }
+  }
+  // tiles wholly on the far side of the diagonal of fixed tile m, and fixed tiles without a token
+  __device__ __forceinline__ bool skip(int m, int i) const {
+    return m >= m_used || (PASS == 1 ? kPfTile * i >= q0 + kPfTile * (m + 1) : i < m);
+  }
+};
+
+// Ring position of one role: index, and the parity of the entry's current use.
+template <int N>
+struct PfRing {
+  int s = 0;
+  uint32_t ph = 0;
+  __device__ __forceinline__ void next() {
+    if (++s == N) {
+      s = 0;
+      ph ^= 1u;
+    }
+  }
+};
+
+// The CTA's items, as one role walks them: the block's own, then the ones launch control handed over. Slot k & 1
+// holds the k-th answer; `leave` lets the slot be refilled (one arrival per role thread or warp).
+struct PfItems {
+  PfRing<2> r;
+  int lin;
+  __device__ __forceinline__ PfItems() : lin((int)blockIdx.x) {}
+  // false: no item is left, or a wait failed
+  __device__ __forceinline__ bool fetch(const PfSmem& sm, volatile int* fail) {
+    if (!pf_wait(sm.ifull(r.s), r.ph, fail)) return false;
+    return launch_answer(sm.item(r.s), lin);
+  }
+  __device__ __forceinline__ void leave(const PfSmem& sm) {
+    fence_proxy_async_smem();  // our read of the answer precedes the next asynchronous write of the slot
+    mbar_arrive(sm.iempty(r.s));
+    r.next();
+  }
+};
+
+// The pipeline shared by both passes. begin() starts an item on an epilogue thread, tile(w, m, i, col0, v, stat)
+// takes its row of one accumulator (columns col0 .. col0 + 31; stat: shared-memory address of those queries'
+// normalisers, pass 2). Two threads share a row, each taking every other tile: put(row) leaves one's partial result in
+// shared memory, end(w, row) joins it to the other's and closes the row. Returns false when a wait timed out (after draining what
+// was in flight); every role leaves through the final barrier.
+template <int MT, int PASS, class Begin, class Tile, class Put, class End>
+__device__ __forceinline__ bool pf_pipeline(const PrefillArgs& a, Begin begin, Tile tile, Put put, End end) {
+  using Work = PfWork<MT, PASS>;
+  constexpr bool STATS = PASS == 2;
+  constexpr int kEpi = 8 * MT, kCopyWarp = kEpi, kMmaWarp = kEpi + 1;  // two MMA warps
+  extern __shared__ uint8_t smem_raw[];
   __shared__ uint32_t s_tmem;
   __shared__ int s_fail;
   volatile int* fail = &s_fail;
-  const PfSmem sm = pf_smem();
+  PfSmem sm;
+  sm.base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const CUtensorMap* map_fix = PASS == 1 ? &a.map_q : &a.map_k;
+  const CUtensorMap* map_str = PASS == 1 ? &a.map_k : &a.map_q;
   if (tid == 0) {
     s_fail = 0;
-    mbar_init(sm.bar_fixed(), 1);
     for (int s = 0; s < kPfStages; ++s) {
       mbar_init(sm.full(s), 1);
-      mbar_init(sm.sfree(s), 1);
-      mbar_init(sm.tfull(s), 1);
-      mbar_init(sm.tempty(s), kPfEpiWarps);  // one arrival per epilogue warp
-      mbar_init(sm.sdone(s), kPfEpiWarps);
+      mbar_init(sm.sfree(s), 2);     // both MMA threads
+      mbar_init(sm.sdone(s), 4 * MT);  // the warps whose turn the tile is
     }
-    mbar_init(sm.drain(), 1);
+    for (int f = 0; f < kPfFix; ++f) {
+      mbar_init(sm.ffull(f), 1);
+      mbar_init(sm.ffree(f), MT == 2 ? 1 : 2);  // the MMA threads that read it
+    }
+    for (int d = 0; d < 4; ++d) {
+      mbar_init(sm.tfull(d), 1);
+      mbar_init(sm.tempty(d), 4);
+    }
+    for (int k = 0; k < 2; ++k) {
+      mbar_init(sm.ifull(k), 1);
+      mbar_init(sm.iempty(k), kEpi + 2);  // the epilogue warps and the MMA threads
+      mbar_init(sm.pfull(k), 4);
+      mbar_init(sm.pempty(k), 4);
+    }
+    mbar_init(sm.drain(), 2);
     fence_mbar_init();
   }
-  if (warp == kPfMmaWarp) tmem_alloc(smem_u32(&s_tmem), kPfTmemCols);
+  if (warp == kCopyWarp && lane == 0) {
+    prefetch_tensormap(map_fix);
+    prefetch_tensormap(map_str);
+  }
+  if (warp == kMmaWarp) tmem_alloc(smem_u32(&s_tmem), kPfTmemCols);
   tcgen05_before_sync();
   __syncthreads();
   tcgen05_after_sync();
   const uint32_t tmem = s_tmem;
 
-  if (warp == kPfCopyWarp) {
-    if (lane == 0) {  // copies: the fixed tile, then the streamed tiles as stages free up
-      int last[kPfStages];
-      for (int s = 0; s < kPfStages; ++s) last[s] = -1;
-      mbar_arrive_expect_tx(sm.bar_fixed(), kPfFixBytes);
-      tma_load_2d(sm.fixed, map_fix, 0, fix_row, sm.bar_fixed());
-      tma_load_2d(sm.fixed + kPfFixHalf, map_fix, 64, fix_row, sm.bar_fixed());
-      for (int t = 0; t < n_tiles; ++t) {
-        const int s = t % kPfStages;
-        const uint32_t ph = ((t / kPfStages) & 1) ^ 1;
-        if (t >= kPfStages && !pf_wait(sm.sfree(s), ph, fail)) break;
-        if (STATS && t >= kPfStages && !pf_wait(sm.sdone(s), ph, fail)) break;
-        const int row = str_row(t);
-        mbar_arrive_expect_tx(sm.full(s), kPfStrBytes + (STATS ? kPfStatBytes : 0));
-        tma_load_2d(sm.stage(s), map_str, 0, row, sm.full(s));
-        tma_load_2d(sm.stage(s) + kPfStrHalf, map_str, 64, row, sm.full(s));
-        if (STATS) bulk_load(sm.stat(s), a.stats + stat_off(t), kPfStatBytes, sm.full(s));
-        last[s] = t;
-      }
-      if (*fail) {  // no copy may outlive the CTA
-        if (!mbar_wait(sm.bar_fixed(), 0)) record_error(a.status, kErrDrainTimeout);
-        for (int s = 0; s < kPfStages; ++s)
-          if (last[s] >= 0 && !mbar_wait(sm.full(s), (last[s] / kPfStages) & 1))
-            record_error(a.status, kErrDrainTimeout);
+  // the copy thread's record of what it has in flight (drained if a wait fails)
+  PfRing<kPfStages> rs;
+  PfRing<kPfFix> rf;
+  int n_str = 0, n_fix = 0;
+  bool asked = false;
+  PfItems items;
+  if (warp == kCopyWarp) {
+    if (lane == 0) {  // next items and copies
+      bool ok = true;
+      for (int k = 0; ok; ++k) {
+        if (k >= 2) ok = pf_wait(sm.iempty(items.r.s), items.r.ph ^ 1u, fail);
+        if (!ok) break;
+        mbar_arrive_expect_tx(sm.ifull(items.r.s), 16);
+        launch_ask(sm.item(items.r.s), sm.ifull(items.r.s));
+        asked = true;
+        const Work w(a, items.lin);
+        const int fix_row = w.head * a.T + w.q0;
+        int m = 0;
+        for (int j = 0; j < w.heads && ok; ++j)
+          for (int i = 0; i < w.n_tiles && ok; ++i) {
+            if (m < MT) {  // the item's fixed tiles go between its first streamed ones (both even if one is unused)
+              const int last = w.heads * w.n_tiles == 1 ? MT : m + 1;
+              for (; m < last && ok; ++m) {
+                if (n_fix >= kPfFix && !(ok = pf_wait(sm.ffree(rf.s), rf.ph ^ 1u, fail))) break;
+                ++n_fix;
+                mbar_arrive_expect_tx(sm.ffull(rf.s), kPfTileBytes);
+                tma_load_2d(sm.fixed(rf.s), map_fix, 0, fix_row + kPfTile * m, sm.ffull(rf.s));
+                tma_load_2d(sm.fixed(rf.s) + kPfHalf, map_fix, 64, fix_row + kPfTile * m, sm.ffull(rf.s));
+                rf.next();
+              }
+              if (!ok) break;
+            }
+            if (n_str >= kPfStages)
+              ok = pf_wait(sm.sfree(rs.s), rs.ph ^ 1u, fail) && (!STATS || pf_wait(sm.sdone(rs.s), rs.ph ^ 1u, fail));
+            if (!ok) break;
+            ++n_str;
+            const int row = w.str_row + j * a.T + kPfTile * i;
+            mbar_arrive_expect_tx(sm.full(rs.s), kPfTileBytes + (STATS ? kPfStatBytes : 0));
+            tma_load_2d(sm.stage(rs.s), map_str, 0, row, sm.full(rs.s));
+            tma_load_2d(sm.stage(rs.s) + kPfHalf, map_str, 64, row, sm.full(rs.s));
+            if (STATS)
+              bulk_load(sm.stat(rs.s), a.stats + (size_t)w.stat_row + (size_t)j * a.T_pad + kPfTile * i, kPfStatBytes,
+                        sm.full(rs.s));
+            rs.next();
+          }
+        if (!ok) break;
+        ok = items.fetch(sm, fail);
+        if (*fail) break;
+        asked = false;
+        items.r.next();  // (this thread refills the slots: it does not count among their readers)
       }
     }
-  } else if (warp == kPfMmaWarp) {
-    if (lane == 0) {  // MMAs: tile n into accumulator n % 4 once its copy landed and its last reader is done
-      if (pf_wait(sm.bar_fixed(), 0, fail)) {
-        for (int n = 0; n < n_tiles; ++n) {
-          const int s = n % kPfStages;
-          const uint32_t ph = (n / kPfStages) & 1;
-          if (!pf_wait(sm.full(s), ph, fail) || !pf_wait(sm.tempty(s), ph ^ 1, fail)) break;
-          tcgen05_after_sync();
-          pf_mma_tile(tmem + (uint32_t)(s * kPfN), sm.fixed, sm.stage(s));
-          umma_commit(sm.sfree(s));
-          umma_commit(sm.tfull(s));
+  } else if (warp == kMmaWarp || warp == kMmaWarp + 1) {
+    if (lane == 0) {  // MMAs: a tile into a free accumulator once its copy landed
+      // MT = 2: the thread multiplies fixed tile p with every streamed tile; MT = 1: the two take turns
+      const int p = warp - kMmaWarp, m = MT == 2 ? p : 0;
+      uint32_t uses = 0;  // accumulator uses of fixed tile m: buffer bit 0, parity bit 1
+      bool ok = true;
+      while (ok) {
+        const Work w(a, items.lin);
+        int f = 0;
+        for (int k = 0; k < MT; ++k) {  // the item's fixed tiles, in order
+          if (k == m) {
+            f = rf.s;
+            ok = pf_wait(sm.ffull(f), rf.ph, fail);
+          }
+          rf.next();
         }
+        for (int j = 0; j < w.heads && ok; ++j)
+          for (int i = 0; i < w.n_tiles && ok; ++i) {
+            ok = pf_wait(sm.full(rs.s), rs.ph, fail);
+            if (ok && !w.skip(m, i)) {
+              const int d = 2 * m + (int)(uses & 1u);
+              if (MT == 2 || (int)(uses & 1u) == p) {
+                ok = pf_wait(sm.tempty(d), ((uses >> 1) & 1u) ^ 1u, fail);
+                if (!ok) break;
+                tcgen05_after_sync();
+                pf_mma_tile(tmem + (uint32_t)(d * kPfTile), sm.fixed(f), sm.stage(rs.s));
+                umma_commit(sm.tfull(d));
+              }
+              ++uses;
+            }
+            if (ok) umma_commit(sm.sfree(rs.s));
+            rs.next();
+          }
+        if (!ok) break;
+        umma_commit(sm.ffree(f));
+        ok = items.fetch(sm, fail);
+        items.leave(sm);
       }
-      umma_commit(sm.drain());  // every MMA issued has completed once this arrives
+      umma_commit(sm.drain());  // every MMA issued has completed once both arrive
       if (!mbar_wait(sm.drain(), 0)) record_error(a.status, kErrDrainTimeout);
     }
-  } else {  // epilogue warps: accumulator lanes 32 (w % 4) .., columns kPfCols (w / 4) ..
-    const int half = warp / 4;
-    for (int n = 0; n < n_tiles; ++n) {
-      const int d = n % kPfAcc;
-      const bool ok = pf_wait(sm.tfull(d), (n / kPfAcc) & 1, fail);
-      if (!__all_sync(0xffffffffu, ok)) {
-        *fail = 1;
-        break;
+  } else {  // epilogue warps: fixed tile m, every other of its accumulators (d = 2 m + p), lanes 32 (w % 4) ..
+    const int m = warp >> 3, p = (warp >> 2) & 1, d = 2 * m + p;
+    const uint32_t acc = tmem + (uint32_t)(d * kPfTile) + ((uint32_t)(32 * (warp & 3)) << 16);
+    const int row = kPfTile * m + 32 * (warp & 3) + lane;
+    uint32_t turn = 0, use = 0, closed = 0;  // whose turn; parities of this accumulator's uses and of the items
+    bool ok = true;
+    while (ok) {
+      const Work w(a, items.lin);
+      begin();
+      for (int j = 0; j < w.heads && ok; ++j)
+        for (int i = 0; i < w.n_tiles; ++i, rs.next()) {
+          const bool skip = w.skip(m, i), mine = (int)turn == p;
+          if (!skip) turn ^= 1u;
+          if (!mine) continue;
+          if (skip) {
+            if (STATS) {  // releases its share of the normalisers; the copy has landed, so this is the stage's phase
+              ok = __all_sync(0xffffffffu, pf_wait(sm.full(rs.s), rs.ph, fail));
+              if (!ok) break;
+              if (lane == 0) mbar_arrive(sm.sdone(rs.s));
+            }
+            continue;
+          }
+          ok = __all_sync(0xffffffffu, pf_wait(sm.tfull(d), use, fail));
+          // the staged normalisers: observe their copy's completion directly (it has completed: the MMAs
+          // that produced this accumulator waited for it, and the stage is not refilled before sdone)
+          if (STATS && ok) ok = __all_sync(0xffffffffu, pf_wait(sm.full(rs.s), rs.ph, fail));
+          if (!ok) break;
+          use ^= 1u;
+          tcgen05_after_sync();
+#pragma unroll 1  // (one copy of the arithmetic: the instruction cache was a limit)
+          for (int c = 0; c < kPfTile; c += kPfCols) {
+            float v[kPfCols];
+            tmem_ld32(acc + c, v);
+            if (c == kPfTile - kPfCols) {  // the accumulator has been read
+              tcgen05_before_sync();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(sm.tempty(d));
+            }
+            tile(w, m, i, c, v, sm.stat(rs.s) + 4 * c);
+            __syncwarp();
+          }
+          if (STATS && lane == 0) mbar_arrive(sm.sdone(rs.s));
+        }
+      if (!ok) break;
+      if (m < w.m_used) {  // the warps of the second accumulator hand their rows' partials to those of the first
+        if (p != 0) {
+          ok = __all_sync(0xffffffffu, pf_wait(sm.pempty(m), closed ^ 1u, fail));
+          if (!ok) break;
+          put(row);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(sm.pfull(m));
+        } else {
+          ok = __all_sync(0xffffffffu, pf_wait(sm.pfull(m), closed, fail));
+          if (!ok) break;
+          end(w, row);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(sm.pempty(m));
+        }
+        closed ^= 1u;
       }
-      tcgen05_after_sync();
-      float v[kPfCols];
-      tmem_ld32(tmem + (uint32_t)(d * kPfN + kPfCols * half) + ((uint32_t)(32 * (warp & 3)) << 16), v);
-      tmem_wait_ld(v);
-      tcgen05_before_sync();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(sm.tempty(d));
-      // the staged normalisers: observe their copy's completion directly (it has completed: the MMAs
-      // that produced this accumulator waited for it, and the stage is not refilled before sdone)
-      if (STATS && !__all_sync(0xffffffffu, pf_wait(sm.full(d), (n / kPfStages) & 1, fail))) {
-        *fail = 1;
-        break;
-      }
-      epi(n, kPfCols * half, v, sm.stat_ptr(d) + kPfCols * half);
-      if (STATS) {
-        __syncwarp();
-        if (lane == 0) mbar_arrive(sm.sdone(d));
+      ok = __all_sync(0xffffffffu, items.fetch(sm, fail));
+      if (lane == 0) {
+        items.leave(sm);
+      } else {
+        items.r.next();
       }
     }
   }
   tcgen05_before_sync();
   __syncthreads();
   const bool failed = s_fail != 0;
-  if (failed && tid == 0) record_error(a.status, kErrFullTimeout);
-  if (warp == kPfMmaWarp) {
+  if (failed) {
+    if (tid == 0) record_error(a.status, kErrFullTimeout);
+    if (warp == kCopyWarp && lane == 0) {  // no copy may outlive the CTA
+      for (int v = 0; v < min(n_str, kPfStages); ++v) {  // the last uses of the ring, latest first
+        rs.ph ^= rs.s == 0 ? 1u : 0u;
+        rs.s = rs.s == 0 ? kPfStages - 1 : rs.s - 1;
+        if (!mbar_wait(sm.full(rs.s), rs.ph)) record_error(a.status, kErrDrainTimeout);
+      }
+      for (int v = 0; v < min(n_fix, kPfFix); ++v) {
+        rf.ph ^= rf.s == 0 ? 1u : 0u;
+        rf.s = rf.s == 0 ? kPfFix - 1 : rf.s - 1;
+        if (!mbar_wait(sm.ffull(rf.s), rf.ph)) record_error(a.status, kErrDrainTimeout);
+      }
+      if (asked && !mbar_wait(sm.ifull(items.r.s), items.r.ph)) record_error(a.status, kErrDrainTimeout);
+    }
+  }
+  if (warp == kMmaWarp) {
     __syncwarp();
     tcgen05_after_sync();
     tmem_dealloc(tmem, kPfTmemCols);
@@ -219,7 +424,15 @@ __device__ __forceinline__ float pf_row_max(const float (&v)[kPfCols]) {
   return fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
 }
 
-// sum_j 2^(v_j * scale - ref): the exponent formed two columns at a time, four independent partial sums.
+// The sum of eight partial sums held as four pairs.
+__device__ __forceinline__ float pf_sum8(const uint64_t (&acc)[4]) {
+  float t[8];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) f32x2_split(acc[k], t[2 * k], t[2 * k + 1]);
+  return ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
+}
+
+// sum_j 2^(v_j * scale - ref): the exponent formed two columns at a time, eight independent partial sums.
 __device__ __forceinline__ float pf_exp_sum(const float (&v)[kPfCols], float scale, float ref) {
   const uint64_t s2 = f32x2(scale, scale), r2 = f32x2(-ref, -ref);
   uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
@@ -229,10 +442,7 @@ __device__ __forceinline__ float pf_exp_sum(const float (&v)[kPfCols], float sca
     f32x2_split(fma_f32x2(f32x2(v[2 * j], v[2 * j + 1]), s2, r2), x0, x1);
     acc[j & 3] = add_f32x2(acc[j & 3], f32x2(fast_exp2(x0), fast_exp2(x1)));
   }
-  float t[8];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) f32x2_split(acc[k], t[2 * k], t[2 * k + 1]);
-  return ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
+  return pf_sum8(acc);
 }
 
 // ------------------------------------------------------------------------------- pass 1: row statistics
@@ -240,124 +450,117 @@ __device__ __forceinline__ float pf_exp_sum(const float (&v)[kPfCols], float sca
 // Per query row the softmax normaliser is accumulated against a reference r (log2 units): the exact maximum
 // of the row's first tile, raised only when a later tile's sum would leave the fp32 range (a logit more than
 // 64 above r, rare), so most tiles need no maximum at all. The pair (r, sum_t 2^(s_t - r)) defines the same
-// normaliser as the true maximum; the kernel stores its log2, r + log2(sum).
+// normaliser as the true maximum; the kernel stores its log2, r + log2(sum), negated (pass 2 adds it).
 
-__global__ void __launch_bounds__(kPfThreads, 2) prefill_rows_kernel(const __grid_constant__ PrefillArgs a) {
-  const int tid = threadIdx.x;
-  const int nq = (a.T + kPfTile - 1) / kPfTile;
-  const int qt = nq - 1 - (int)blockIdx.x;  // the longest rows first
-  const int bq = blockIdx.y;                // b * Hq + query head
-  const int G = a.heads_q / a.heads_kv;
-  const int b = bq / a.heads_q, h = (bq - b * a.heads_q) / G;
-  const int krow0 = (b * a.heads_kv + h) * a.T;
-  __shared__ float s_r[kPfTile], s_l[kPfTile];  // the second column half's partial of each row
-  const int row = tid & (kPfTile - 1);
-  const int q = kPfTile * qt + row;  // an epilogue thread's query
-  const int kend = min(kPfTile * (qt + 1), a.T);  // keys 0 .. kend - 1 can reach this tile's queries
-  float r = -INFINITY, l = 0.f;  // over this thread's column half of every tile
-  const bool ok = pf_pipeline<false>(
-      a, &a.map_q, bq * a.T + kPfTile * qt, &a.map_k_str, (kend + kPfN - 1) / kPfN,
-      [&](int n) { return krow0 + kPfN * n; }, [](int) { return (size_t)0; },
-      [&](int n, int col0, float (&v)[kPfCols], const float*) {
-        const int k0 = kPfN * n + col0;
-        if (k0 + kPfCols > kPfTile * qt) {  // keys after the query, or past the prefill, do not count
+template <int MT>
+__global__ void __launch_bounds__(pf_threads(MT), 1) prefill_rows_kernel(const __grid_constant__ PrefillArgs a) {
+  using Work = PfWork<MT, 1>;
+  __shared__ float s_r[MT * kPfTile], s_l[MT * kPfTile];  // one thread's partial of each row
+  float r = -INFINITY, l = 0.f;                           // over this thread's tiles
+  pf_pipeline<MT, 1>(
+      a,
+      [&] {
+        r = -INFINITY;
+        l = 0.f;
+      },
+      [&](const Work& w, int m, int i, int col0, float (&v)[kPfCols], uint32_t) {
+        const int k0 = kPfTile * i + col0;
+        if (k0 + kPfCols > w.q0 + kPfTile * m) {  // keys after the query do not count
+          const int q = w.q0 + kPfTile * m + (int)(threadIdx.x & 127u);
 #pragma unroll
           for (int j = 0; j < kPfCols; ++j)
-            if (k0 + j > q || k0 + j >= a.T) v[j] = -INFINITY;
-        }
-        if (r == -INFINITY) {  // the row's first tile fixes the reference
-          const float mx = pf_row_max(v);
-          if (mx == -INFINITY) return;
-          r = mx * a.scale_log2;
+            if (k0 + j > q) v[j] = -INFINITY;
         }
         float sum = pf_exp_sum(v, a.scale_log2, r);
-        if (!(sum <= 0x1p64f)) {  // a logit far above the reference: move the reference to this tile's maximum
-          const float rn = fmaxf(r, pf_row_max(v) * a.scale_log2);
-          sum = pf_exp_sum(v, a.scale_log2, rn);
-          l *= fast_exp2(r - rn);
+        // the row's first columns (r = -inf), or a logit far above the reference: move the reference to the maximum
+        if (__any_sync(0xffffffffu, !(sum <= 0x1p64f))) {
+          float rn = r;
+          if (!(sum <= 0x1p64f)) rn = fmaxf(r, pf_row_max(v) * a.scale_log2);
+          sum = rn == -INFINITY ? 0.f : pf_exp_sum(v, a.scale_log2, rn);
+          if (rn != r) l *= fast_exp2(r - rn);
           r = rn;
         }
         l += sum;
+      },
+      [&](int row) {
+        s_r[row] = r;
+        s_l[row] = l;
+      },
+      [&](const Work& w, int row) {  // both partials against the larger reference
+        const int q = w.q0 + row;
+        const float r2 = s_r[row], rm = fmaxf(r, r2);
+        const float lt = (r == -INFINITY ? 0.f : l * fast_exp2(r - rm)) +
+                         (r2 == -INFINITY ? 0.f : s_l[row] * fast_exp2(r2 - rm));
+        a.stats[(size_t)w.head * a.T_pad + q] = q < a.T ? -(rm + log2f(lt)) : -INFINITY;
       });
-  if (tid >= kPfTile && tid < 2 * kPfTile) {
-    s_r[row] = r;
-    s_l[row] = l;
-  }
-  __syncthreads();
-  if (ok && tid < kPfTile) {  // both halves against the larger reference
-    const float r2 = s_r[row], rm = fmaxf(r, r2);
-    const float lt = (r == -INFINITY ? 0.f : l * fast_exp2(r - rm)) + (r2 == -INFINITY ? 0.f : s_l[row] * fast_exp2(r2 - rm));
-    a.stats[(size_t)bq * a.T_pad + q] = q < a.T ? rm + log2f(lt) : INFINITY;
-  }
 }
 
 // ------------------------------------------------------------------------------ pass 2: column sums
 
-__global__ void __launch_bounds__(kPfThreads, 2) prefill_cols_kernel(const __grid_constant__ PrefillArgs a) {
-  const int tid = threadIdx.x;
-  const int kt = blockIdx.x;  // the keys with the most queries first
-  const int bh = blockIdx.y;  // b * Hkv + KV head
-  const int G = a.heads_q / a.heads_kv;
-  const int b = bh / a.heads_kv, h = bh - b * a.heads_kv;
-  const int per_head = (a.T - kPfTile * kt + kPfN - 1) / kPfN;  // query tiles of each head reaching the keys
-  // query tile n: head j = n / per_head, first query kPfTile kt + kPfN (n % per_head)
-  auto qhead = [&](int n) { return b * a.heads_q + h * G + n / per_head; };
-  auto qfirst = [&](int n) { return kPfTile * kt + kPfN * (n % per_head); };
-  __shared__ float s_cs[kPfTile];  // the second column half's sum of each row
-  const int row = tid & (kPfTile - 1);
-  const int key = kPfTile * kt + row;  // an epilogue thread's key
+template <int MT>
+__global__ void __launch_bounds__(pf_threads(MT), 1) prefill_cols_kernel(const __grid_constant__ PrefillArgs a) {
+  using Work = PfWork<MT, 2>;
+  __shared__ float s_cs[MT * kPfTile];  // one thread's sum of each row
   float cs = 0.f;
-  const bool ok = pf_pipeline<true>(
-      a, &a.map_k, bh * a.T + kPfTile * kt, &a.map_q_str, G * per_head,
-      [&](int n) { return qhead(n) * a.T + qfirst(n); },
-      [&](int n) { return (size_t)qhead(n) * a.T_pad + qfirst(n); },
-      [&](int n, int col0, float (&v)[kPfCols], const float* stat) {
-        const int q0 = qfirst(n) + col0;
-        // the log2 normalisers of these queries, staged with the tile (+inf for padding: they weigh nothing)
-        const float4* nc = reinterpret_cast<const float4*>(stat);
-        if (q0 < kPfTile * (kt + 1)) {  // the diagonal: queries before the key do not attend to it
+  pf_pipeline<MT, 2>(
+      a, [&] { cs = 0.f; },
+      [&](const Work& w, int m, int i, int col0, float (&v)[kPfCols], uint32_t stat) {
+        const int q0 = w.q0 + kPfTile * i + col0;
+        // minus the log2 normalisers of these queries, staged with the tile (-inf for padding: they weigh nothing)
+        uint32_t c[kPfCols / 4][4];
+#pragma unroll
+        for (int j = 0; j < kPfCols / 4; ++j) lds_vec<4>(stat + 16 * j, c[j]);
+        // queries before the key do not attend to it; rows past the prefill belong to another head
+        if (i == m || q0 + kPfCols > a.T) {
+          const int key = w.q0 + kPfTile * m + (int)(threadIdx.x & 127u);
 #pragma unroll
           for (int j = 0; j < kPfCols; ++j)
-            if (q0 + j < key) v[j] = -INFINITY;
+            if (q0 + j < key || q0 + j >= a.T) v[j] = -INFINITY;
         }
         const uint64_t s2 = f32x2(a.scale_log2, a.scale_log2);
         uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll
-        for (int j = 0; j < kPfCols / 4; ++j) {
-          const float4 c = nc[j];
-          float x0, x1, x2, x3;
-          f32x2_split(fma_f32x2(f32x2(v[4 * j], v[4 * j + 1]), s2, f32x2(-c.x, -c.y)), x0, x1);
-          f32x2_split(fma_f32x2(f32x2(v[4 * j + 2], v[4 * j + 3]), s2, f32x2(-c.z, -c.w)), x2, x3);
-          acc[(2 * j) & 3] = add_f32x2(acc[(2 * j) & 3], f32x2(fast_exp2(x0), fast_exp2(x1)));
-          acc[(2 * j + 1) & 3] = add_f32x2(acc[(2 * j + 1) & 3], f32x2(fast_exp2(x2), fast_exp2(x3)));
+        for (int j = 0; j < kPfCols / 2; ++j) {
+          float x0, x1;
+          f32x2_split(fma_f32x2(f32x2(v[2 * j], v[2 * j + 1]), s2,
+                                f32x2(__uint_as_float(c[j / 2][2 * (j & 1)]), __uint_as_float(c[j / 2][2 * (j & 1) + 1]))),
+                      x0, x1);
+          acc[j & 3] = add_f32x2(acc[j & 3], f32x2(fast_exp2(x0), fast_exp2(x1)));
         }
-        float t[8];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) f32x2_split(acc[k], t[2 * k], t[2 * k + 1]);
-        cs += ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
+        cs += pf_sum8(acc);
+      },
+      [&](int row) { s_cs[row] = cs; },
+      [&](const Work& w, int row) {
+        if (w.q0 + row < a.T) a.scores[(size_t)w.head * a.T + w.q0 + row] = cs + s_cs[row];
       });
-  if (tid >= kPfTile && tid < 2 * kPfTile) s_cs[row] = cs;
-  __syncthreads();
-  if (ok && tid < kPfTile && key < a.T) a.scores[(size_t)bh * a.T + key] = cs + s_cs[row];
+}
+
+template <int MT>
+cudaError_t pf_launch(PrefillArgs a, cudaStream_t st) {
+  static bool configured = false;
+  if (!configured) {
+    cudaError_t e = cudaFuncSetAttribute(prefill_rows_kernel<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPfSmem);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(prefill_cols_kernel<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPfSmem);
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
+  const int items = (a.T + MT * kPfTile - 1) / (MT * kPfTile);
+  const int per = (2 * kPfSlots + items - 1) / items;  // heads per group: about two rounds of the resident CTAs
+  a.group_rows = a.group_cols = per;
+  prefill_rows_kernel<MT><<<items * a.batch * a.heads_q, pf_threads(MT), kPfSmem, st>>>(a);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  prefill_cols_kernel<MT><<<items * a.batch * a.heads_kv, pf_threads(MT), kPfSmem, st>>>(a);
+  return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_prefill(const PrefillArgs& a, int batch, cudaStream_t st) {
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(prefill_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPfSmem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(prefill_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPfSmem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
-  const int nt = (a.T + kPfTile - 1) / kPfTile;
-  prefill_rows_kernel<<<dim3(nt, batch * a.heads_q), kPfThreads, kPfSmem, st>>>(a);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  prefill_cols_kernel<<<dim3(nt, batch * a.heads_kv), kPfThreads, kPfSmem, st>>>(a);
-  return cudaGetLastError();
+// Items of two fixed tiles when they fill the GPU, else of one: a small prefill then has twice the CTAs.
+cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st) {
+  const int items2 = (a.T + 2 * kPfTile - 1) / (2 * kPfTile);
+  return (long long)items2 * a.batch * a.heads_kv >= kPfSlots ? pf_launch<2>(a, st) : pf_launch<1>(a, st);
 }
 
 }  // namespace mikv

@@ -61,6 +61,29 @@ def test_prefill_scores_match_oracle(B, Hq, Hkv, T):
     np.testing.assert_allclose(got.sum(axis=2), G * T, rtol=rtol)  # every query row's weights sum to one
 
 
+@pytest.mark.parametrize("T", [1, 127, 128, 129, 255, 256, 257, 385])
+@pytest.mark.parametrize("B,Hq,Hkv", [(20, 16, 8), (3, 4, 2)], ids=["items256", "items128"])
+def test_prefill_scores_tile_edges(B, Hq, Hkv, T):
+    """Lengths around the 128-token tiles, with enough heads for items of two fixed tiles and with few: an item whose
+    second tile has no, one or all tokens, streamed tiles that end inside a tile, and (many items per block) the
+    hand-over from one item to the next. One head is scaled up and the next one down, so that rows read past a head's
+    end would show."""
+    w = mi.Workload("pfe", B, Hq, Hkv, T, 1, 2, 32, 0.2, seed=T + Hq)
+    k, _ = mi.prefill_kv(w, 0)
+    q = mi.prefill_queries(w, 0)
+    q[:, ::2] *= 4
+    k[:, 1::2] *= 0.25
+    got = _gpu_scores(w, q, k)
+    G = Hq // Hkv
+    assert np.all(np.isfinite(got))
+    for b, h in [(0, 0), (B // 2, 1), (B - 1, Hkv - 1)]:
+        qh, kh = bits16(q[b:b + 1, h * G:(h + 1) * G]), bits16(k[b:b + 1, h:h + 1])
+        ref = oracle.prefill_scores(qh, kh, 1 / math.sqrt(128))[0, 0]
+        np.testing.assert_allclose(got[b, h], ref, rtol=prefill_rtol(qh, kh, T, G), atol=1e-30)
+    rtol = prefill_rtol(bits16(q), bits16(k), T, G)
+    np.testing.assert_allclose(got.sum(axis=2), G * T, rtol=rtol)
+
+
 @pytest.mark.parametrize("B,Hq,Hkv,T,heads", [(8, 32, 32, 4096, [(0, 0), (7, 31)]),   # Llama-2-7B shape
                                               (2, 32, 8, 8192, [(1, 5)])],           # GQA, G = 4
                          ids=["llama2-7b-t4096", "gqa4-t8192"])
