@@ -95,6 +95,17 @@ __device__ __forceinline__ uint32_t eq1_code_exact(float x, const Eq1Params& p) 
   return (uint32_t)(c < 0 ? 0 : (c > QMAX ? QMAX : c));
 }
 
+// The same decision for a pair of values in packed fp32 (Eq. 1 of both): y holds 2^23 + code in each half, whose low
+// 16 bits are the code, and off the two distances from the nearest integer. For finite values no clamp is needed:
+// x >= beta, and alpha >= (1 - 2^-23) span / QMAX, so the product rounds into [0, QMAX]; the others have an
+// infinite or NaN distance and are re-decided.
+__device__ __forceinline__ void eq1_pair_fast(uint64_t x, uint64_t neg_beta, uint64_t ralpha, uint64_t& y,
+                                              uint64_t& off) {
+  const uint64_t q = mul_f32x2(add_f32x2(x, neg_beta), ralpha);
+  y = add_f32x2(q, f32x2(8388608.f, 8388608.f));
+  off = fma_f32x2(add_f32x2(y, f32x2(-8388608.f, -8388608.f)), f32x2(-1.f, -1.f), q);  // q - rint(q), exact
+}
+
 // Quantize one row (Eq. 1) held as fp32 values x[4] of channels 4 lane .. 4 lane + 3 of each lane, with
 // one warp. Writes 16 * BITS bytes of packed codes to `codes` (8-byte aligned) and 128 / GROUP
 // (alpha, beta) fp16 pairs to `params`. Every rounding is explicit (fsub/fdiv round-to-nearest, fp16
