@@ -53,30 +53,86 @@ __device__ int block_exclusive_scan(int v, int* total, int* sh) {
   return before;
 }
 
-// One block per (b, h): the n_demote smallest keys leave; both lists come out in ascending index order.
+// The 32-bit halves of order_key: scores and ids as unsigned integers of the same order.
+__device__ __forceinline__ uint32_t score_key(float s) { return (uint32_t)(order_key(s, 0) >> 32); }
+__device__ __forceinline__ uint32_t id_key(int32_t id) { return (uint32_t)(id ^ (int32_t)0x80000000); }
+
+// The value of rank `rank` (from 0) among key(i) of the entries with take(i), i < n: three radix passes of 11, 11 and
+// 10 bits from the top. Leaves the value, its rank among its equals and how many equals there are.
+struct Ranked {
+  uint32_t value;
+  int rank, equals;
+};
+constexpr int kBins = 2 * kSelThreads;  // two bins per thread in the search for the digit
+
+template <class Key, class Take>
+__device__ Ranked radix_rank(int n, int rank, Key key, Take take, unsigned int* hist, int* sh, Ranked* s_out) {
+  const int tid = threadIdx.x;
+  uint32_t prefix = 0, mask = 0;
+  int equals = 0;
+#pragma unroll 1
+  for (int pass = 0; pass < 3; ++pass) {
+    const int shift = pass == 0 ? 21 : pass == 1 ? 10 : 0;
+    const uint32_t digits = pass == 2 ? 0x3ffu : 0x7ffu;
+    hist[tid] = 0u;
+    hist[tid + kSelThreads] = 0u;
+    __syncthreads();
+#pragma unroll 4
+    for (int i = tid; i < n; i += kSelThreads) {
+      const uint32_t k = key(i);
+      if ((k & mask) == prefix && take(i)) atomicAdd(&hist[(k >> shift) & digits], 1u);
+    }
+    __syncthreads();
+    const int c0 = (int)hist[2 * tid], c1 = (int)hist[2 * tid + 1];
+    int total;
+    const int before = block_exclusive_scan(c0 + c1, &total, sh);
+    if (rank >= before && rank < before + c0 + c1) {  // exactly one thread
+      const bool second = rank >= before + c0;
+      s_out->value = prefix | ((uint32_t)(2 * tid + second) << shift);
+      s_out->rank = rank - before - (second ? c0 : 0);
+      s_out->equals = second ? c1 : c0;
+    }
+    __syncthreads();
+    prefix = s_out->value;
+    rank = s_out->rank;
+    equals = s_out->equals;
+    mask |= digits << shift;
+    __syncthreads();
+  }
+  return {prefix, rank, equals};
+}
+
+// One block per (b, h): the n_demote smallest keys leave; both lists come out in ascending index order. Bound by
+// latency and by the L2 reads of the scores (five or six of n x 4 bytes), so the passes are few and wide: the score
+// alone is ranked first (three 11-bit passes, the digit found by a block scan), the id only among scores equal to the
+// last one demoted, and the lists are written with coalesced stores from one scan of the warps' counts. (Eight
+// byte-wide passes over (score, id), each with a serial search for the digit, and lists written a run per thread took
+// 163 us for 256 heads of 32768 scores; this takes 49.)
+constexpr int kSelRounds = 32;  // rounds of kSelThreads entries whose choice a thread keeps in one register
+
 __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* scores, const int32_t* ids, int n,
                                                              int stride, int n_demote, int32_t* demoted,
                                                              int32_t* kept) {
-  __shared__ unsigned int hist[256];
+  __shared__ unsigned int hist[kBins];
   __shared__ int sh[64];
+  __shared__ int s_off[kSelRounds * (kSelThreads / 32)];
   __shared__ unsigned long long s_best[kSelThreads / 32];
-  __shared__ unsigned long long s_prefix;
-  __shared__ int s_rank;
-  const int bh = blockIdx.x, tid = threadIdx.x;
+  __shared__ Ranked s_ranked;
+  const int bh = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const float* sc = scores + (size_t)bh * stride;
   const int32_t* id = ids ? ids + (size_t)bh * stride : nullptr;
   int32_t* dem = demoted + (size_t)bh * n_demote;
   int32_t* kep = kept ? kept + (size_t)bh * (n - n_demote) : nullptr;
+  auto ident = [&](int i) { return id ? id[i] : i; };
 
-  unsigned long long thresh;  // largest key that is demoted
-  if (n_demote == 0) {
-    thresh = 0ull;  // nothing demoted (keys are never 0: the top bit of a score key is set or ~)
-  } else if (n_demote == n) {
-    thresh = ~0ull;
+  // the largest key that is demoted, by its halves (keys are never 0: the top bit of a score key is set or ~)
+  uint32_t last_score = 0u, last_id = 0u;
+  if (n_demote == n) {
+    last_score = last_id = ~0u;
   } else if (n_demote == 1) {
     unsigned long long best = ~0ull;
     for (int i = tid; i < n; i += kSelThreads) {
-      const unsigned long long k = order_key(sc[i], id ? id[i] : i);
+      const unsigned long long k = order_key(sc[i], ident(i));
       best = k < best ? k : best;
     }
 #pragma unroll
@@ -84,69 +140,68 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* scores
       const unsigned long long o = __shfl_xor_sync(0xffffffffu, best, off);
       best = o < best ? o : best;
     }
-    if ((tid & 31) == 0) s_best[tid >> 5] = best;
+    if (lane == 0) s_best[warp] = best;
     __syncthreads();
-    if (tid < 32) {
-      best = tid < kSelThreads / 32 ? s_best[tid] : ~0ull;
+    best = s_best[lane];
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        const unsigned long long o = __shfl_xor_sync(0xffffffffu, best, off);
-        best = o < best ? o : best;
-      }
-      if (tid == 0) s_prefix = best;
+    for (int off = 16; off > 0; off >>= 1) {
+      const unsigned long long o = __shfl_xor_sync(0xffffffffu, best, off);
+      best = o < best ? o : best;
     }
-    __syncthreads();
-    thresh = s_prefix;
-  } else {
-    // Radix select of the key of rank n_demote - 1, 8 bits per pass from the top.
-    unsigned long long prefix = 0ull;
-    int rank = n_demote - 1;
-    for (int pass = 0; pass < 8; ++pass) {
-      const int shift = 56 - 8 * pass;
-      const unsigned long long hi_mask = pass == 0 ? 0ull : (~0ull << (shift + 8));
-      for (int i = tid; i < 256; i += kSelThreads) hist[i] = 0u;
-      __syncthreads();
-      for (int i = tid; i < n; i += kSelThreads) {
-        const unsigned long long k = order_key(sc[i], id ? id[i] : i);
-        if ((k & hi_mask) == prefix) atomicAdd(&hist[(k >> shift) & 0xffu], 1u);
-      }
-      __syncthreads();
-      if (tid == 0) {
-        int acc = 0, dgt = 0;
-        for (; dgt < 256; ++dgt) {
-          if (acc + (int)hist[dgt] > rank) break;
-          acc += (int)hist[dgt];
-        }
-        s_prefix = prefix | ((unsigned long long)dgt << shift);
-        s_rank = rank - acc;
-      }
-      __syncthreads();
-      prefix = s_prefix;
-      rank = s_rank;
-      __syncthreads();
-    }
-    thresh = prefix;
+    last_score = (uint32_t)(best >> 32);
+    last_id = (uint32_t)best;
+  } else if (n_demote > 1) {
+    const Ranked s = radix_rank(n, n_demote - 1, [&](int i) { return score_key(sc[i]); }, [](int) { return true; }, hist,
+                                sh, &s_ranked);
+    last_score = s.value;
+    last_id = ~0u;
+    if (s.rank + 1 < s.equals)  // only some of the equal scores leave: those with the smallest ids
+      last_id = radix_rank(n, s.rank, [&](int i) { return id_key(ident(i)); },
+                           [&](int i) { return score_key(sc[i]) == last_score; }, hist, sh, &s_ranked)
+                    .value;
   }
 
-  // Ascending-index compaction: thread tid owns indices [tid * per, (tid + 1) * per).
-  const int per = (n + kSelThreads - 1) / kSelThreads;
-  const int i0 = tid * per, i1 = min(n, i0 + per);
-  int cnt = 0;
-  for (int i = i0; i < i1; ++i) cnt += order_key(sc[i], id ? id[i] : i) <= thresh && n_demote > 0;
-  int total;
-  int pos = block_exclusive_scan(cnt, &total, sh);
-  int kpos = i0 - pos;
-  for (int i = i0; i < i1; ++i) {
-    const bool d = n_demote > 0 && order_key(sc[i], id ? id[i] : i) <= thresh;
-    if (d) {
-      if (pos < n_demote) dem[pos] = i;
-      ++pos;
-    } else {
-      if (kep && kpos < n - n_demote) kep[kpos] = i;
-      ++kpos;
+  // ascending-index lists: the choices of up to kSelRounds rounds (bit k of `out`), the warps' counts scanned, then
+  // every entry written to its place
+  int base = 0;  // demoted before these rounds
+  for (int i0 = 0; i0 < n; i0 += kSelRounds * kSelThreads) {
+    uint32_t out = 0u;
+#pragma unroll 4
+    for (int k = 0; k < kSelRounds; ++k) {
+      const int i = i0 + k * kSelThreads + tid;
+      bool d = false;
+      if (i < n && n_demote > 0) {
+        const uint32_t s = score_key(sc[i]);
+        d = s < last_score || (s == last_score && (last_id == ~0u || id_key(ident(i)) <= last_id));
+      }
+      const uint32_t votes = __ballot_sync(0xffffffffu, d);
+      out |= (uint32_t)d << k;
+      if (lane == 0) s_off[k * (kSelThreads / 32) + warp] = __popc(votes);
     }
+    __syncthreads();
+    int total;
+    const int before = block_exclusive_scan(s_off[tid], &total, sh);  // (leaves through a block barrier)
+    s_off[tid] = base + before;
+    base += total;
+    __syncthreads();
+#pragma unroll 4
+    for (int k = 0; k < kSelRounds; ++k) {
+      const int i = i0 + k * kSelThreads + tid;
+      const bool d = (out >> k) & 1u;
+      const uint32_t votes = __ballot_sync(0xffffffffu, d);
+      const int pos = s_off[k * (kSelThreads / 32) + warp] + __popc(votes & ((1u << lane) - 1u));  // demoted before i
+      if (i < n) {
+        if (d) {
+          if (pos < n_demote) dem[pos] = i;
+        } else if (kep && i - pos < n - n_demote) {
+          kep[i - pos] = i;
+        }
+      }
+    }
+    __syncthreads();
   }
 }
+static_assert(kSelRounds * (kSelThreads / 32) == kSelThreads, "one warp count per thread in the scan");
 
 __global__ void __launch_bounds__(64) insert_kernel(__nv_bfloat16* k_hi, __nv_bfloat16* v_hi, int32_t* hi_tok,
                                                     float* acc, const __nv_bfloat16* k_new,
