@@ -28,6 +28,7 @@ __all__ = [
 ]
 
 HEAD_DIM = 128
+FILL_WHOLE = 32 << 20
 OUT_BF16, OUT_F32 = 0, 1
 WS_ATTENTION, WS_BALANCER, WS_STEP, WS_PREFILL = 0, 1, 2, 3
 STATUS = {0: "MIKV_OK", 1: "MIKV_ERR_ARG", 2: "MIKV_ERR_UNSUPPORTED", 3: "MIKV_ERR_CAPACITY",
@@ -167,32 +168,46 @@ def shape_for_context(batch: int, heads_q: int, heads_kv: int, bits: int, group:
 class LayerCache:
     """Device arrays of one layer's mixed-precision cache (allocated by torch; layouts of mikv_cache)."""
 
-    def __init__(self, shape: Shape, device="cuda", balancer: torch.Tensor = None):
+    def __init__(self, shape: Shape, device="cuda", balancer: torch.Tensor = None, filled=None):
+        """filled = (important rows, retained tokens) that the caller writes next in every head: of an array of
+        FILL_WHOLE bytes or more only the other rows are then zeroed (zeroing everything first wrote a whole cache
+        once more: 0.40 of the 3.45 ms build of the batch-32, 32768-token Mistral-7B layer). Below that a fill of the
+        whole array takes the GPU less time (5 us for 32 MiB) than the extra slice takes the host."""
         s = shape
         B, H, d = s.batch, s.heads_kv, s.head_dim
         self.shape = s
-        z = dict(device=device)
+        hi, lo = filled if filled is not None else (0, 0)
+        if s.k_channel_group:  # the incomplete last group of retained tokens goes to the staging rows
+            lo = lo // s.k_channel_group * s.k_channel_group
+
+        def rows(n, first, *tail, dtype):  # [B, H, n, *tail], zero from row `first` on
+            if not first or B * H * n * math.prod(tail) * dtype.itemsize < FILL_WHOLE:
+                return torch.zeros(B, H, n, *tail, dtype=dtype, device=device)
+            t = torch.empty(B, H, n, *tail, dtype=dtype, device=device)
+            t[:, :, first:].zero_()
+            return t
+
         if s.hi_coded:  # codes of balanced keys / values plus (alpha, beta) per group
-            self.k_hi = torch.zeros(B, H, s.hi_stride, 16 * s.hi_bits, dtype=torch.uint8, **z)
-            self.v_hi = torch.zeros(B, H, s.hi_stride, 16 * s.hi_bits, dtype=torch.uint8, **z)
-            self.k_hi_params = torch.zeros(B, H, s.hi_stride, d // s.hi_group, 2, dtype=torch.float16, **z)
-            self.v_hi_params = torch.zeros(B, H, s.hi_stride, d // s.hi_group, 2, dtype=torch.float16, **z)
+            self.k_hi = rows(s.hi_stride, hi, 16 * s.hi_bits, dtype=torch.uint8)
+            self.v_hi = rows(s.hi_stride, hi, 16 * s.hi_bits, dtype=torch.uint8)
+            self.k_hi_params = rows(s.hi_stride, hi, d // s.hi_group, 2, dtype=torch.float16)
+            self.v_hi_params = rows(s.hi_stride, hi, d // s.hi_group, 2, dtype=torch.float16)
         else:
-            self.k_hi = torch.zeros(B, H, s.hi_stride, d, dtype=torch.bfloat16, **z)
-            self.v_hi = torch.zeros(B, H, s.hi_stride, d, dtype=torch.bfloat16, **z)
+            self.k_hi = rows(s.hi_stride, hi, d, dtype=torch.bfloat16)
+            self.v_hi = rows(s.hi_stride, hi, d, dtype=torch.bfloat16)
             self.k_hi_params = self.v_hi_params = None
-        self.hi_tok = torch.zeros(B, H, s.hi_stride, dtype=torch.int32, **z)
-        self.acc = torch.zeros(B, H, s.hi_stride, dtype=torch.float32, **z)
+        self.hi_tok = rows(s.hi_stride, hi, dtype=torch.int32)
+        self.acc = rows(s.hi_stride, hi, dtype=torch.float32)
         # (bits = 0: eviction, no retained set; its arrays are empty)
-        self.k_codes = torch.zeros(B, H, s.lo_cap, 16 * s.bits, dtype=torch.uint8, **z)
-        self.v_codes = torch.zeros(B, H, s.lo_cap, 16 * s.bits, dtype=torch.uint8, **z)
+        self.k_codes = rows(s.lo_cap, lo, 16 * s.bits, dtype=torch.uint8)
+        self.v_codes = rows(s.lo_cap, lo, 16 * s.bits, dtype=torch.uint8)
         npar = d // s.group if s.bits else 0
         if s.k_channel_group:  # one (alpha, beta) per channel and group of 64 retained tokens
-            self.k_params = torch.zeros(B, H, s.lo_cap // s.k_channel_group, d, 2, dtype=torch.float16, **z)
+            self.k_params = rows(s.lo_cap // s.k_channel_group, lo // s.k_channel_group, d, 2, dtype=torch.float16)
         else:
-            self.k_params = torch.zeros(B, H, s.lo_cap, npar, 2, dtype=torch.float16, **z)
-        self.v_params = torch.zeros(B, H, s.lo_cap, npar, 2, dtype=torch.float16, **z)
-        self.lo_tok = torch.zeros(B, H, s.lo_cap, dtype=torch.int32, **z)
+            self.k_params = rows(s.lo_cap, lo, npar, 2, dtype=torch.float16)
+        self.v_params = rows(s.lo_cap, lo, npar, 2, dtype=torch.float16)
+        self.lo_tok = rows(s.lo_cap, lo, dtype=torch.int32)
         self.balancer = balancer
         self.n_lo = 0
 

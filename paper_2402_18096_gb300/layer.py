@@ -28,9 +28,9 @@ def workspace(nbytes: int, device="cuda") -> torch.Tensor:
 class MixedPrecisionLayer:
     """One layer's MiKV cache plus the per-step state (free slots, retained length, workspace)."""
 
-    def __init__(self, shape: Shape, balancer: torch.Tensor = None, device="cuda"):
+    def __init__(self, shape: Shape, balancer: torch.Tensor = None, device="cuda", filled=None):
         self.shape = shape
-        self.cache = LayerCache(shape, device=device, balancer=balancer)
+        self.cache = LayerCache(shape, device=device, balancer=balancer, filled=filled)
         self.slots = torch.zeros(shape.batch, shape.heads_kv, dtype=torch.int32, device=device)
         self.ws = workspace(mikv_workspace_bytes(shape, WS_STEP, shape.lo_cap), device)
         self.n_lo = 0
@@ -57,8 +57,8 @@ class MixedPrecisionLayer:
             bal = torch.empty(H, shape.head_dim, dtype=torch.float32, device=device)
             ws = workspace(mikv_workspace_bytes(shape, WS_BALANCER, 0), device)
             mikv_compute_balancer(shape, q_pre, k, bal, ws)
-        layer = cls(shape, balancer=bal, device=device)
         n_demote = T - k_budget
+        layer = cls(shape, balancer=bal, device=device, filled=(k_budget, n_demote if shape.bits else 0))
         demoted = torch.empty(B, H, n_demote, dtype=torch.int32, device=device)
         kept = torch.empty(B, H, k_budget, dtype=torch.int32, device=device)
         mikv_select_demote(scores, T, n_demote, demoted, kept)

@@ -1,12 +1,13 @@
 """GPU parity of the cache-build kernels at the edges of their tiles: the bulk quantizer's rounds, the balancer's
-row chunks and its path for unaligned inputs, the bulk selection's rounds and ties, the gather's row groups.
-Everything here is bit-exact."""
+row chunks and its path for unaligned inputs, the bulk selection's rounds and ties, the gather's row groups, and the
+rows a build leaves zero. Everything here is bit-exact."""
 import numpy as np
 import pytest
 import torch
 
 import oracle
 import paper_2402_18096_gb300 as pkg
+from paper_2402_18096_gb300.layer import MixedPrecisionLayer
 from _cases import bits16, new_workspace
 
 pytestmark = pytest.mark.gpu
@@ -144,3 +145,26 @@ def test_gather_row_counts(n_rows, aligned):
     ref["hi_tok"][1, 1, 0] = ref["acc"][1, 1, 0] = 0
     np.testing.assert_array_equal(cache.hi_tok[:, :, :n_rows].cpu().numpy(), ref["hi_tok"][:, :, :n_rows])
     np.testing.assert_array_equal(cache.acc[:, :, :n_rows].cpu().numpy(), ref["acc"][:, :, :n_rows])
+
+
+@pytest.mark.parametrize("bits,hi_bits,kch", [(2, 16, 0), (3, 8, 0), (2, 16, 64), (0, 16, 0)],
+                         ids=["bf16", "coded", "per-channel", "evict"])
+def test_build_zeroes_what_it_does_not_write(bits, hi_bits, kch, monkeypatch):
+    """A build that zeroes only the rows it does not write leaves the same arrays as one that zeroes everything."""
+    gen = torch.Generator().manual_seed(9)
+    B, H, T = 2, 2, 333
+    dev = torch.device("cuda")
+    k, v = _rand_bf16(B, H, T, D, gen=gen).to(dev), _rand_bf16(B, H, T, D, gen=gen).to(dev)
+    scores = torch.rand(B, H, T, generator=gen).to(dev)
+    shape = pkg.shape_for_context(B, H, H, bits, 32, T, 0.2, 40, hi_bits=hi_bits, k_channel_group=kch)
+    built = []
+    for whole in (1 << 60, 0):
+        monkeypatch.setattr(pkg, "FILL_WHOLE", whole)
+        junk = torch.full((64 << 20,), 0xFF, dtype=torch.uint8, device=dev)  # what the allocator hands out next
+        del junk
+        cache = MixedPrecisionLayer.from_prefill(shape, k, v, scores, device=dev).cache
+        built.append({n: t.clone() for n, t in vars(cache).items() if isinstance(t, torch.Tensor)})
+    for name, want in built[0].items():
+        got = built[1][name]
+        as_bytes = lambda t: t.contiguous().view(torch.uint8) if t.numel() else t  # noqa: E731
+        assert torch.equal(as_bytes(got), as_bytes(want)), name
