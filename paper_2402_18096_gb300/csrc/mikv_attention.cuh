@@ -274,24 +274,43 @@ __device__ __forceinline__ uint32_t code8(uint32_t r, int hi) {
   return exact_codes(prmt(r, 0x64646464u, hi ? 0x4341u : 0x4240u), 0x64006400u);
 }
 
-// 3-bit code with its low bits at [p, p + 2) of r and its high bit at p + 2 of hs (each unit), OR-ed under
-// `magic`, the fp16 exponent that makes bit p weigh 1: the pair holds magic + code exactly. In the 1-bit plane
-// the bits of the two channels u and u + 8 of a unit alternate (bit 2 m + (u div 8) for channel 16 m + u), so
-// one shift of the plane word lines up the high bit of every code of a channel with its low bits.
-__device__ __forceinline__ uint32_t or_code3(uint32_t r, uint32_t hs, int p, uint32_t magic) {
-  return and_or(hs, 0x00040004u << p, and_or(r, 0x00030003u << p, magic));
+// 3-bit codes. A register r of the 2-bit plane holds the low bits of code m of each unit at [2m, 2m + 2), and a word
+// of the 1-bit plane the codes' high bits, those of the two channels u and u + 8 of a unit by turns (bit 2m + (u div
+// 8)): one shift of the plane word lines up the high bit of every code of a channel two bits above its low bits. There
+// it collides with the low bits of the next code, so the codes are merged by turns, each set with one bit-select:
+//   e = codes 0, 2 at bits 0, 4 and o = codes 1, 3 at bits 2, 6   (r, plane word << 2, or << 1 for channels u + 8)
+//   e8, o8: the same of codes 4, 6 and 5, 7                       (r >> 8, plane word >> 6, or >> 7)
+// with a bit of the other plane's neighbour left between them, which the extraction mask drops. A code pair then costs
+// one LOP3, where merging it alone cost two (136 ALU instructions per 16-token block instead of 168; the blocks are
+// bound by the ALU pipe: Llama-2-13B step 164.9 -> 153.1 us, batch-64 INT3 g128 5 % attention 239 -> 220 us, INT3 on the
+// Mistral-7B shape 281.6 -> 265.9 us).
+struct Merged3 {
+  uint32_t e, o, e8, o8;
+  __device__ __forceinline__ Merged3(uint32_t r, uint32_t plane, bool high) {  // high: channels u + 8
+    const uint32_t r8 = r >> 8, h = high ? plane << 1 : plane << 2, h8 = high ? plane >> 7 : plane >> 6;
+    e = bit_select(r, h, 0x33333333u);
+    o = bit_select(r, h, 0xCCCCCCCCu);
+    e8 = bit_select(r8, h8, 0x33333333u);
+    o8 = bit_select(r8, h8, 0xCCCCCCCCu);
+  }
+  // the word of code m and, in it, the code's position: 0, 2, 4 or 6
+  __device__ __forceinline__ uint32_t word(int m) const { return m < 4 ? (m & 1 ? o : e) : (m & 1 ? o8 : e8); }
+  static __host__ __device__ constexpr int pos(int m) { return 4 * ((m >> 1) & 1) + 2 * (m & 1); }
+};
+
+// Key codes (exact) of k-step ks, N = 3.
+__device__ __forceinline__ uint32_t kcode3(const Merged3& x, int ks) {
+  const int p = Merged3::pos(ks);
+  return exact_codes(and_or(x.word(ks), 0x00070007u << p, mag2(p / 2)), mag2(p / 2));
 }
 
-// Key codes (exact) of k-step ks, N = 3: kr = a fragment register of the 2-bit plane (its codes for ks at bits
-// 2 ks), kr8 = kr >> 8; he / he8 the 1-bit plane word shifted so that the high bits of ks <= 3 / ks >= 4 land
-// at 2 ks + 2 / 2 (ks - 4) + 2.
-__device__ __forceinline__ uint32_t kcode3(uint32_t kr, uint32_t kr8, uint32_t he, uint32_t he8, int ks) {
-  const int j = ks & 3;
-  return exact_codes(or_code3(ks < 4 ? kr : kr8, ks < 4 ? he : he8, 2 * j, mag2(j)), mag2(j));
+// Value codes, N = 3, take a code offset M in {64, 16} like vcode2: code mt is read at bit 4 + 2 (mt & 1), its word
+// shifted there when it sits at bit 0 or 2.
+__device__ __forceinline__ uint32_t vcode3(const Merged3& x, int mt) {
+  const uint32_t w = Merged3::pos(mt) < 4 ? x.word(mt) << 4 : x.word(mt);
+  const int p = 4 + 2 * (mt & 1);
+  return and_or(w, 0x00070007u << p, mag2(p / 2));
 }
-
-// Value codes, N = 3, take a code offset M in {64, 16} like vcode2: code mt is read at bit 4 + 2 (mt & 1) of the
-// words shifted by 4 - 4 (mt div 2) (the low bits) and by two more (the high bit).
 __host__ __device__ constexpr float voff3(int mt) { return (mt & 1) ? 16.f : 64.f; }
 
 // Value codes (N = 2, 4) skip the subtraction: the code is placed at a mantissa position where it
@@ -328,12 +347,11 @@ template <int BITS, int PITCH>
 struct KeyFrag {
   static constexpr int NR = BITS == 4 ? 8 : 4;
   uint32_t kr[NR], kh[NR];
-  uint32_t he0, he1, ho0, ho1, he0s, he1s, ho0s, ho1s;  // N = 3 only
+  uint32_t kb0 = 0, kb1 = 0;  // N = 3: the 1-bit plane words of tokens g and g + 8
 
   __device__ __forceinline__ void load(uint32_t rows, int lane) {
     const int r8 = lane & 7, j = lane >> 3;
     const int tok = r8 + 8 * (j & 1);
-    uint32_t kb0 = 0, kb1 = 0;
     if (BITS == 4) {
       const int o0 = tok * 64 + 16 * (j >> 1), sw = ((tok >> 1) & 3) << 4;
       uint32_t r0[4], r1[4];
@@ -355,11 +373,6 @@ struct KeyFrag {
     }
 #pragma unroll
     for (int i = 0; i < NR; ++i) kh[i] = kr[i] >> (BITS == 2 ? 10 : 8);
-    // N = 3: the 1-bit plane words of tokens g (kb0) and g + 8 (kb1) shifted so that the high bit of code ks sits
-    // two bits above its low bits: channels 2t, 2t+1 use the even bits (<< 2 for ks <= 3, >> 6 for ks >= 4),
-    // channels 2t+8, 2t+9 the odd bits (<< 1, >> 7)
-    he0 = kb0 << 2, he1 = kb1 << 2, ho0 = kb0 << 1, ho1 = kb1 << 1;
-    he0s = kb0 >> 6, he1s = kb1 >> 6, ho0s = kb0 >> 7, ho1s = kb1 >> 7;
   }
 
   // exact codes of k-step ks (channels 16 ks .. 16 ks + 15) as fp16 pairs
@@ -372,10 +385,12 @@ struct KeyFrag {
 #pragma unroll
       for (int i = 0; i < 4; ++i) c[i] = code2(kr[i], kh[i], ks);
     } else {
-      c[0] = kcode3(kr[0], kh[0], he0, he0s, ks);
-      c[1] = kcode3(kr[1], kh[1], he1, he1s, ks);
-      c[2] = kcode3(kr[2], kh[2], ho0, ho0s, ks);
-      c[3] = kcode3(kr[3], kh[3], ho1, ho1s, ks);
+      // kr[0], kr[1]: channels 2t, 2t + 1 of tokens g, g + 8; kr[2], kr[3]: channels 2t + 8, 2t + 9 (the merged words
+      // are shared by all k-steps)
+      c[0] = kcode3(Merged3(kr[0], kb0, false), ks);
+      c[1] = kcode3(Merged3(kr[1], kb1, false), ks);
+      c[2] = kcode3(Merged3(kr[2], kb0, true), ks);
+      c[3] = kcode3(Merged3(kr[3], kb1, true), ks);
     }
   }
 };
@@ -433,15 +448,11 @@ struct ValFrag {
           a[i] = vcode2(vr[i] << 4, vr[i], vr[i] >> 6, mt);  // the shifted copies are shared by all mt
       }
     } else {
-      // vr[0], vr[2]: channel g (tokens 2t, 2t+1 and 2t+8, 2t+9), whose high bits are the even bits of vb0, vb1;
-      // vr[1], vr[3]: channel g + 8, the odd bits
-      const int k = mt >> 1, s = 4 - 4 * k;  // codes 2k, 2k+1 read at bits 4, 6 of the words shifted by s
-      auto sh = [](uint32_t x, int n) { return n >= 0 ? x << n : x >> -n; };
-      const uint32_t r4[4] = {sh(vr[0], s), sh(vr[1], s), sh(vr[2], s), sh(vr[3], s)};
-      const uint32_t h4[4] = {sh(vb0, s + 2), sh(vb0, s + 1), sh(vb1, s + 2), sh(vb1, s + 1)};
-      const int p = 4 + 2 * (mt & 1);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = or_code3(r4[i], h4[i], p, mag2(p >> 1));
+      // vr[0], vr[2]: channel g (tokens 2t, 2t+1 and 2t+8, 2t+9); vr[1], vr[3]: channel g + 8
+      a[0] = vcode3(Merged3(vr[0], vb0, false), mt);
+      a[1] = vcode3(Merged3(vr[1], vb0, true), mt);
+      a[2] = vcode3(Merged3(vr[2], vb1, false), mt);
+      a[3] = vcode3(Merged3(vr[3], vb1, true), mt);
     }
   }
 };
