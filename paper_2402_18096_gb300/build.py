@@ -11,6 +11,7 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -22,6 +23,7 @@ LIB_DEBUG = os.path.join(OUT_DIR_DEBUG, "libmikv_debug.so")
 SOURCES = ["mikv_attn_h16.cu", "mikv_attn_h8.cu", "mikv_attn_h4.cu", "mikv_attn_h2.cu", "mikv_attn_kch.cu",
            "mikv_attention.cu",
            "mikv_quant.cu", "mikv_policy.cu", "mikv_step.cu", "mikv_prefill.cu", "mikv_abi.cu"]
+PYCALL = "mikv_pycall.c"  # the binding's decode-path calls as an extension module (where Python's headers are installed)
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 
@@ -35,9 +37,30 @@ def _nvcc() -> str:
 
 def _inputs():
     files = [os.path.join(CSRC, s) for s in SOURCES]
-    files += [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
+    files += [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h", ".c"))]
     files.append(os.path.join(os.path.dirname(HERE), "include", "mikv.h"))
     return files
+
+
+def pycall_path(debug: bool = False) -> str:
+    return os.path.join(OUT_DIR_DEBUG if debug else OUT_DIR, "mikv_pycall.so")
+
+
+def _build_pycall(debug: bool) -> None:
+    """The extension module, or none (and no stale one) without Python's headers or a C compiler."""
+    out = pycall_path(debug)
+    include = sysconfig.get_paths()["include"]
+    gcc = shutil.which("gcc") or shutil.which("cc")
+    if not gcc or not os.path.exists(os.path.join(include, "Python.h")):
+        if os.path.exists(out):
+            os.unlink(out)
+        return
+    tmp = out + f".tmp{os.getpid()}"
+    cmd = [gcc, "-O2", "-std=c11", "-shared", "-fPIC", "-Wall", "-I", include, os.path.join(CSRC, PYCALL), "-o", tmp]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"{gcc} failed on {PYCALL}:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, out)
 
 
 def up_to_date(debug: bool = False) -> bool:
@@ -66,6 +89,7 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
             print(r.stdout, r.stderr, file=sys.stderr)
         return obj
 
+    _build_pycall(debug)
     with ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
         objs = list(ex.map(compile_one, SOURCES))
     tmp = lib + f".tmp{os.getpid()}"
