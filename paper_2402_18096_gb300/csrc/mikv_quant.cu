@@ -27,6 +27,7 @@ struct QPArgs {
   int32_t* lo_tok;
   int* dbg;  // debug builds: the library's status word for index checks (nullptr otherwise)
   int heads_kv, n_src, n_rows, lo_start, lo_cap;
+  int rounds;  // rounds of a block
 };
 
 // Bulk quantize/pack (Eq. 1): eight lanes per row and four rows per warp. Lane l8 = lane & 7 of a row owns
@@ -36,100 +37,83 @@ struct QPArgs {
 // them turns into whole words, one or two per lane.
 // It is bound by instruction issue (a row's bytes move in a third of the time its scalar arithmetic took), so the
 // arithmetic is packed: pairs of channels in fp32x2, minima and maxima three at a time, the code taken from the
-// rounded sum's low bits without a clamp, the doubtful codes found by one maximum over the lane's channels. A warp
-// walks kQpRounds x 16 rows with the balancer in registers and the next rows' loads in flight behind the
-// arithmetic. B 32, Hkv 8, 26214 rows of K and V each, INT2 g32: 1839 -> 1275 us (the bytes at the copy rate: 600).
+// rounded sum's low bits without a clamp, the doubtful codes found by one maximum over the lane's channels, the words
+// joined on the FMA pipe. A warp walks several rounds of rows with the next rows' loads in flight behind the
+// arithmetic; the balancer waits in shared memory, which leaves 60 registers and four blocks per SM (70 registers and
+// three blocks: 1230 us). B 32, Hkv 8, 26214 rows of K and V each, INT2 g32: 1839 -> 1086 us (the bytes at the copy
+// rate: 600).
 constexpr int kQpRowsPerWarp = 4;
-constexpr int kQpRounds = 8;                          // rounds of a block (16 rows of K and of V each)
-constexpr int kQpBlockRows = 4 * kQpRowsPerWarp;      // rows of a round
+constexpr int kQpBlockRows = 4 * kQpRowsPerWarp;      // rows of a round (16 of K and of V each)
+constexpr int kQpRoundsMax = 16;
+constexpr int kQpBlocks = 2 * 152 * 4;                // fewer rounds per block until the grid has this many blocks
 
-// Reduce-scatter of N partial words over lane bits OFF, OFF / 2, ...: in each round a lane keeps the half
-// of its words selected by its lane bit and ORs in the partner's copy of that half. After log2(N) rounds
-// lane l8 holds the whole word index (bits of l8 from OFF down), as a single value.
-template <int N, int OFF>
-__device__ __forceinline__ uint32_t reduce_scatter(const uint32_t (&w)[N], int l8) {
-  constexpr int H = N / 2;
-  const bool up = (l8 & OFF) != 0;
-  uint32_t k[H];
+// Packs one row's codes: w[k] = code of channel 16 l8 + 2 k | code of channel 16 l8 + 2 k + 1 << 16. A word of the row
+// collects the same k from the lanes that share it, so the row's words are transposed through the warp's shared memory
+// (x: word k of lane l at 8 k + l, rows 72 words apart: no bank conflicts) and joined by multiply-adds, which the FMA
+// pipe takes where selects, shifts and shuffles loaded the ALU pipe.
+constexpr int kQpRowWords = 72;
+
+template <int N>
+__device__ __forceinline__ uint32_t join_fields(const uint32_t* x, uint32_t step) {  // sum of x[m] step^m
+  uint32_t v = x[N - 1];
 #pragma unroll
-  for (int i = 0; i < H; ++i) {
-    const uint32_t send = up ? w[i] : w[i + H];
-    k[i] = (up ? w[i + H] : w[i]) | __shfl_xor_sync(0xffffffffu, send, OFF);
-  }
-  if constexpr (H == 1) {
-    return k[0];
-  } else {
-    return reduce_scatter<H, OFF / 2>(k, l8);
-  }
+  for (int m = N - 2; m >= 0; --m) v = v * step + x[m];
+  return v;
 }
 
-// Stores one row's codes (low bits of the pairs w[k] = code of channel 16 l8 + 2 k | channel 16 l8 + 2 k + 1 << 16).
 template <int BITS>
-__device__ __forceinline__ void qp_store_codes(const uint32_t (&w)[8], uint32_t* row, int l8, bool valid) {
+__device__ __forceinline__ void qp_store_codes(const uint32_t (&w)[8], uint32_t* x, uint32_t* row, int l8, bool valid) {
+  __syncwarp();  // (the previous round's words have been read)
+#pragma unroll
+  for (int k = 0; k < 8; ++k) x[8 * k + l8] = w[k];
+  __syncwarp();
+  uint32_t f[8];
   if constexpr (BITS == 4) {
-    // channel 16 l8 + u: unit 16 (l8 >> 2) + u, bits 4 (l8 & 3); the lanes with equal l8 >> 2 share
-    // words 8 (l8 >> 2) .. + 7, and lane l8 ends with words 2 l8, 2 l8 + 1
-    const int sh = 4 * (l8 & 3);
-    uint32_t L[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) L[k] = w[k] << sh;
-    uint32_t K[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const bool up = (l8 & 2) != 0;
-      K[k] = (up ? L[k + 4] : L[k]) | __shfl_xor_sync(0xffffffffu, up ? L[k] : L[k + 4], 2);
-    }
-    uint32_t out[2];
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const bool up = (l8 & 1) != 0;
-      out[k] = (up ? K[k + 2] : K[k]) | __shfl_xor_sync(0xffffffffu, up ? K[k] : K[k + 2], 1);
-    }
-    if (valid) *reinterpret_cast<uint2*>(row + 2 * l8) = make_uint2(out[0], out[1]);
+    // channel 16 l8 + u: unit 16 (l8 >> 2) + u, bits 4 (l8 & 3); lane l8 writes words 2 l8 and 2 l8 + 1, each joined
+    // from four lanes
+    const uint4* p = reinterpret_cast<const uint4*>(x + 8 * ((2 * l8) & 7) + 4 * (l8 >> 2));
+    const uint4 a = p[0], b = p[2];
+    const uint32_t fa[4] = {a.x, a.y, a.z, a.w}, fb[4] = {b.x, b.y, b.z, b.w};
+    if (valid) *reinterpret_cast<uint2*>(row + 2 * l8) = make_uint2(join_fields<4>(fa, 16u), join_fields<4>(fb, 16u));
   } else {
-    // two-bit fields (INT2, and the low bits of INT3): channel 16 l8 + u sits in unit u at bits 2 l8;
-    // all eight lanes share words 0..7, and lane l8 ends with word l8
-    uint32_t L[8];
+    // two-bit fields (INT2, and the low bits of INT3): channel 16 l8 + u sits in unit u at bits 2 l8: lane l8 writes
+    // word l8
+    const uint4* p = reinterpret_cast<const uint4*>(x + 8 * l8);
+    const uint4 a = p[0], b = p[1];
+    const uint32_t g[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
-    for (int k = 0; k < 8; ++k) L[k] = (BITS == 3 ? w[k] & 0x00030003u : w[k]) << (2 * l8);
-    const uint32_t wd = reduce_scatter<8, 4>(L, l8);
-    if (valid) row[l8] = wd;
+    for (int m = 0; m < 8; ++m) f[m] = BITS == 3 ? g[m] & 0x00030003u : g[m];
+    if (valid) row[l8] = join_fields<8>(f, 4u);
     if constexpr (BITS == 3) {
-      // high bits: channel 16 l8 + u sits in unit u & 7 at bit 2 l8 + (u >> 3) (words 8..11 of the row);
-      // after two rounds a lane pair holds one word, and the pair's even lane stores it
-      uint32_t H[4];
+      // high bits: channel 16 l8 + u sits in unit u & 7 at bit 2 l8 + (u >> 3) (words 8..11 of the row): lanes l8 and
+      // l8 + 4 hold the even and the odd bits of a word
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
-        H[k] = (((w[k] >> 2) & 0x00010001u) | ((w[k + 4] >> 1) & 0x00020002u)) << (2 * l8);
-      uint32_t K[2];
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const bool up = (l8 & 4) != 0;
-        K[k] = (up ? H[k + 2] : H[k]) | __shfl_xor_sync(0xffffffffu, up ? H[k] : H[k + 2], 4);
-      }
-      const bool up = (l8 & 2) != 0;
-      uint32_t hw = (up ? K[1] : K[0]) | __shfl_xor_sync(0xffffffffu, up ? K[0] : K[1], 2);
-      hw |= __shfl_xor_sync(0xffffffffu, hw, 1);
-      if (valid && (l8 & 1) == 0) row[8 + (l8 >> 1)] = hw;
+      for (int m = 0; m < 8; ++m) f[m] = g[m] & 0x00040004u;
+      const uint32_t h = (f[0] >> 2) + join_fields<7>(f + 1, 4u);  // (bit 2 of field m at bit 2 m)
+      const uint32_t o = __shfl_xor_sync(0xffffffffu, h, 4);
+      if (valid && l8 < 4) row[8 + l8] = h | (o << 1);
     }
   }
 }
 
 template <int BITS, int GROUP>
-__global__ void __launch_bounds__(256) quantize_pack_kernel(const QPArgs a) {
+__global__ void __launch_bounds__(256, 4) quantize_pack_kernel(const QPArgs a) {
   constexpr int QMAX = (1 << BITS) - 1;
   constexpr int GL = GROUP / 16;  // lanes per quantization group
+  __shared__ __align__(16) uint32_t s_words[8][4 * kQpRowWords];
+  __shared__ float4 s_bal[kHeadDim / 4];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, l8 = lane & 7;
   const bool is_v = (w & 1) != 0;
   const int bh = blockIdx.y, h = bh % a.heads_kv;
   const int32_t* rows = a.rows + (size_t)bh * a.n_rows;
   const __nv_bfloat16* src = (is_v ? a.v_src : a.k_src) + (size_t)bh * a.n_src * kHeadDim + 16 * l8;
-  const int i0 = blockIdx.x * (kQpRounds * kQpBlockRows) + (w >> 1) * kQpRowsPerWarp + (lane >> 3);
+  const int i0 = blockIdx.x * (a.rounds * kQpBlockRows) + (w >> 1) * kQpRowsPerWarp + (lane >> 3);
   const bool balanced = !is_v && a.balancer;  // Eq. 3: keys times the balancer before the quantizer (warp-uniform)
-  float4 bal[4];
-  if (balanced) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) bal[k] = reinterpret_cast<const float4*>(a.balancer + h * kHeadDim + 16 * l8)[k];
+  // the head's balancer in shared memory: piece k of lane l8 at 8 k + l8 (no bank conflicts)
+  if (a.balancer) {
+    if (threadIdx.x < 32)
+      s_bal[8 * (lane & 3) + (lane >> 2)] = reinterpret_cast<const float4*>(a.balancer + h * kHeadDim)[lane];
+    __syncthreads();
   }
   // row i of this lane, -1 past the end; an out-of-range source row is skipped (documented in the ABI)
   auto row_of = [&](int i) { return i < a.n_rows ? rows[i] : -1; };
@@ -145,7 +129,7 @@ __global__ void __launch_bounds__(256) quantize_pack_kernel(const QPArgs a) {
   uint4 raw[2];
   load(r, raw);
 #pragma unroll 1
-  for (int t = 0; t < kQpRounds; ++t) {
+  for (int t = 0; t < a.rounds; ++t) {
     const int i = i0 + t * kQpBlockRows;
     if (__all_sync(0xffffffffu, i >= a.n_rows)) break;
     const bool valid = in_range(r);
@@ -159,15 +143,16 @@ __global__ void __launch_bounds__(256) quantize_pack_kernel(const QPArgs a) {
     }
     // the next round's rows, behind this round's arithmetic
     const int rn = r_next;
-    if (t + 1 < kQpRounds) {
+    if (t + 1 < a.rounds) {
       load(rn, raw);
-      r_next = t + 2 < kQpRounds ? row_of(i + 2 * kQpBlockRows) : -1;
+      r_next = t + 2 < a.rounds ? row_of(i + 2 * kQpBlockRows) : -1;
     }
     if (balanced) {
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        x[2 * k] = mul_f32x2(x[2 * k], f32x2(bal[k].x, bal[k].y));
-        x[2 * k + 1] = mul_f32x2(x[2 * k + 1], f32x2(bal[k].z, bal[k].w));
+        const float4 b = s_bal[8 * k + l8];
+        x[2 * k] = mul_f32x2(x[2 * k], f32x2(b.x, b.y));
+        x[2 * k + 1] = mul_f32x2(x[2 * k + 1], f32x2(b.z, b.w));
       }
     }
     float mn, mx;
@@ -210,9 +195,9 @@ __global__ void __launch_bounds__(256) quantize_pack_kernel(const QPArgs a) {
         wd[k] = eq1_code_exact<QMAX>(lo, p) | (eq1_code_exact<QMAX>(hi, p) << 16);
       }
     }
-    __syncwarp();
     const size_t pos = (size_t)bh * a.lo_cap + a.lo_start + i;
-    qp_store_codes<BITS>(wd, reinterpret_cast<uint32_t*>((is_v ? a.v_codes : a.k_codes) + pos * (16 * BITS)), l8, valid);
+    qp_store_codes<BITS>(wd, s_words[w] + kQpRowWords * (lane >> 3),
+                         reinterpret_cast<uint32_t*>((is_v ? a.v_codes : a.k_codes) + pos * (16 * BITS)), l8, valid);
     if (valid && l8 % GL == 0)
       ((is_v ? a.v_params : a.k_params) + pos * (kHeadDim / GROUP))[(16 * l8) / GROUP] =
           __halves2half2(p.alpha16, p.beta16);
@@ -537,7 +522,9 @@ cudaError_t launch_quantize_pack(const mikv_shape& s, const mikv_cache& c, const
   a.n_rows = n_rows;
   a.lo_start = lo_start;
   a.lo_cap = s.lo_cap;
-  const int per_block = kQpRounds * kQpBlockRows;
+  const long long all = (long long)((n_rows + kQpBlockRows - 1) / kQpBlockRows) * s.batch * s.heads_kv;  // rounds in all
+  a.rounds = (int)(all / kQpBlocks < 1 ? 1 : all / kQpBlocks < kQpRoundsMax ? all / kQpBlocks : kQpRoundsMax);
+  const int per_block = a.rounds * kQpBlockRows;
   const dim3 grid((n_rows + per_block - 1) / per_block, s.batch * s.heads_kv);
   switch (s.bits) {
     case 2: return qp_group<2>(a, s.group, grid, st);
