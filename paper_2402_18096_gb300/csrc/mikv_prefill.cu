@@ -14,9 +14,11 @@
 //
 // What bounds it: one exponential per score and pass (32 per clock and SM: 512 clocks per 128 x 128 tile) weighs as
 // much as the tile's MMAs (512 clocks at the tensor peak), so both have to run all the time.
-//  - Two warps issue MMAs, one per fixed tile. The issuing thread is held while its MMAs run and then spends about
-//    450 clocks on the hand-over (measured: 0, 4, 8 and 16 MMAs a tile took 446, 726, 993 and 1466 clocks), so one
-//    thread alone leaves the tensor cores idle half of the time; the other's MMAs fill its gap.
+//  - Two warps issue MMAs, one per fixed tile. A thread takes 46 clocks to issue an MMA and some 450 for the hand-over
+//    of a tile (measured: 0, 4, 8 and 16 MMAs a tile took 446, 726, 993 and 1466 clocks), so one thread alone leaves the
+//    tensor cores idle half of the time; the other's MMAs fill its gap. (N = 256 keeps them full from one thread, 1025
+//    clocks for eight MMAs, but then two accumulators fill the tensor memory and all sixteen epilogue warps share
+//    each: 1086 against 1022 us for the whole call below.)
 //  - Two accumulators per fixed tile, so that MMAs run under the arithmetic, and one streamed tile for two fixed ones
 //    (MT = 2), which halves the traffic from L2 per score (the 128-row tiles drew 7.9 TB/s).
 //  - Four sets of four epilogue warps, one set per accumulator, each warp taking whole rows of 128 columns: a hand-over
@@ -557,7 +559,10 @@ cudaError_t pf_launch(PrefillArgs a, cudaStream_t st) {
 
 }  // namespace
 
-// Items of two fixed tiles when they fill the GPU, else of one: a small prefill then has twice the CTAs.
+// Items of two fixed tiles when pass 2 then still has one per SM (its items are the fewer ones), else of one, which
+// gives a small prefill twice the CTAs. Either side measured, one tile against two: Hkv 8, T 4864 (152 items of two
+// tiles) 280.9 / 248.5 us, T 3000 (96) 151.1 / 155.0 us, T 2048 (64) 84.5 / 99.9 us, T 8192 (256) 749 / 599 us;
+// H 32, T 608, B 2 (192) 32.8 / 29.2 us, T 512, B 1 (64) 20.6 / 21.0 us.
 cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st) {
   const int items2 = (a.T + 2 * kPfTile - 1) / (2 * kPfTile);
   return (long long)items2 * a.batch * a.heads_kv >= kPfSlots ? pf_launch<2>(a, st) : pf_launch<1>(a, st);
