@@ -36,8 +36,24 @@ __device__ __forceinline__ float merge_weight(const float* part_ml, int G, int b
 
 __device__ __forceinline__ void merge_stats_warp(const float* part_ml, int G, int bh, int jh, int w0, int w1, int lane,
                                                  float& M, float& L) {
+  constexpr float kLog2e = 1.4426950408889634f;
   const int n = w1 - w0 + 1;
   M = -INFINITY;
+  if (n <= 32) {  // one read of (max, sum) per partial; the arithmetic below, term by term
+    float ms = -INFINITY, ls = 0.f;
+    if (lane < n) {
+      const float2 v = __ldcg(reinterpret_cast<const float2*>(part_ml + ((size_t)(w0 + lane + bh) * G + jh) * 2));
+      ms = v.x;
+      ls = v.y;
+    }
+    M = ms;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
+    L = ms != -INFINITY ? fast_exp2((ms - M) * kLog2e) * ls : 0.f;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) L += __shfl_xor_sync(0xffffffffu, L, off);
+    return;
+  }
   for (int c0 = 0; c0 < n; c0 += 32) {
     const int i = c0 + lane;
     if (i < n) M = fmaxf(M, part_ml[((size_t)(w0 + i + bh) * G + jh) * 2]);
@@ -88,14 +104,17 @@ __device__ __forceinline__ void merge_output_warp(const float* part_o, const flo
 
 // Both steps at once when the head has at most NB partials: every load (each partial's statistics and output)
 // is issued before any is used, so the merge costs one round of loads; the arithmetic, and its order, is that of
-// merge_stats_warp followed by merge_output_warp, so the bits are the same. More partials take those two.
-template <int NB>
+// merge_stats_warp followed by merge_output_warp, so the bits are the same. More partials take those two. on_stats()
+// is called as soon as M and L are known.
+template <int NB, class OnStats>
 __device__ __forceinline__ void merge_head_warp(const float* part_o, const float* part_ml, int G, int bh, int jh,
-                                                int w0, int w1, int lane, float& M, float& L, float (&out)[4]) {
+                                                int w0, int w1, int lane, float& M, float& L, float (&out)[4],
+                                                OnStats on_stats) {
   constexpr float kLog2e = 1.4426950408889634f;
   const int n = w1 - w0 + 1;
   if (n > NB || n > 32) {
     merge_stats_warp(part_ml, G, bh, jh, w0, w1, lane, M, L);
+    on_stats();
     merge_output_warp(part_o, part_ml, G, bh, jh, w0, w1, lane, M, L, out);
     return;
   }
@@ -117,6 +136,7 @@ __device__ __forceinline__ void merge_head_warp(const float* part_o, const float
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) Lp += __shfl_xor_sync(0xffffffffu, Lp, off);
   L = Lp;
+  on_stats();
   float O[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
   for (int k = 0; k < NB; ++k) {
