@@ -78,6 +78,7 @@ constexpr int kThreads = kWarps * 32;
 constexpr int kNS = MIKV_ATTN_STAGES;       // ring stages per warp
 constexpr bool kLoPair = MIKV_LO_PAIR != 0;  // retained blocks processed two at a time
 constexpr int kPairAcc = MIKV_PAIR_ACC;      // QK^T accumulators per block when paired
+constexpr int kStageBytes = kUnitBytes;
 constexpr int kHiBlockBytes = 8192;         // K and V of 16 tokens: 4 boxes of 16 rows x 64 bf16
 constexpr int kCtasPerSm = MIKV_ATTN_CTAS;
 constexpr int kQkAcc = MIKV_QK_ACC;         // independent accumulators of the QK^T MMA chain
@@ -85,9 +86,7 @@ constexpr int kUnitsPerWarp = 24;    // share the grid sizing starts from; the p
                                      // it can (min(units, slots) warps)
 constexpr float kLog2e = 1.4426950408889634f;
 
-__host__ __device__ constexpr int smem_bytes(int hi_bits) {
-  return 1024 + kWarps * kNS * stage_bytes(hi_bits) + kWarps * kNS * 8;
-}
+__host__ __device__ constexpr int smem_bytes() { return 1024 + kWarps * kNS * kStageBytes + kWarps * kNS * 8; }
 
 // Position in the concatenated unit sequence. Unit i of a head (of n_u units, hu of them important)
 // is important when floor((i+1) hu / n_u) > floor(i hu / n_u): important units are spread evenly.
@@ -1202,7 +1201,6 @@ template <int BITS, int GROUP, int HB, int G, bool KCH = false>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm) attention_kernel(const __grid_constant__ AttnArgs a) {
   constexpr LoUnit U = KCH ? lo_unit_layout_kch(BITS, GROUP) : lo_unit_layout(BITS, GROUP);
   constexpr LoUnit H = lo_unit_layout(HB == 16 ? 2 : HB, kHiGroup);
-  constexpr int kStageBytes = stage_bytes(HB);
   static_assert(U.total <= kStageBytes && H.total <= kStageBytes, "unit too large for a stage");
   static_assert(!KCH || HB == 16, "per-channel retained keys need a bf16 important set");
   // one query head per KV head with a bf16 important set and per-token retained keys: the group-column path
@@ -1444,7 +1442,7 @@ template <int BITS, int GROUP, int HB, int G, bool KCH = false>
 cudaError_t launch_kernel(const AttnArgs& a, int grid, cudaStream_t st) {
   auto kern = attention_kernel<BITS, GROUP, HB, G, KCH>;
   static bool configured = false;
-  const int smem = smem_bytes(HB);
+  const int smem = smem_bytes();
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;

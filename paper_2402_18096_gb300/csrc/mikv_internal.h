@@ -79,16 +79,10 @@ __host__ __device__ constexpr LoUnit lo_unit_layout_kch(int bits, int group) {
   return u;
 }
 
-// Bytes of a ring stage by the precision of the important set. INT8 important rows take 4352 bytes a block: a stage of
-// 9216 holds two, which are then taken together (one block alone has nothing to overlap with: batch-32 Mistral-7B
-// shape, INT8 important, step 240.6 -> 232.7 us). With the other sets larger stages gained on some shapes what they
-// lost on others (INT2 g32: Mistral-7B 250.6 -> 252.9, at 5 % important 223.5 -> 217.8 us).
-__host__ __device__ constexpr int stage_bytes(int hi_bits) { return hi_bits == 8 ? 9216 : kUnitBytes; }
-
-// The largest unit (at most 8 blocks) that fits one stage (8-bit codes are those of an important set).
+// The largest unit (at most 8 blocks) that fits one stage.
 __host__ __device__ constexpr LoUnit lo_unit_layout(int bits, int group) {
   int n = 8;
-  while (n > 1 && lo_unit_layout_n(bits, group, n).total > stage_bytes(bits)) --n;
+  while (n > 1 && lo_unit_layout_n(bits, group, n).total > kUnitBytes) --n;
   return lo_unit_layout_n(bits, group, n);
 }
 
