@@ -205,7 +205,7 @@ __device__ __forceinline__ bool pf_pipeline(const PrefillArgs& a, Begin begin, T
     }
     for (int f = 0; f < kPfFix; ++f) {
       mbar_init(sm.ffull(f), 1);
-      mbar_init(sm.ffree(f), MT == 2 ? 1 : 2);  // the MMA threads that read it
+      mbar_init(sm.ffree(f), 2);     // both MMA threads
     }
     for (int d = 0; d < 4; ++d) {
       mbar_init(sm.tfull(d), 1);
@@ -290,11 +290,20 @@ __device__ __forceinline__ bool pf_pipeline(const PrefillArgs& a, Begin begin, T
       bool ok = true;
       while (ok) {
         const Work w(a, items.lin);
-        int f = 0;
-        for (int k = 0; k < MT; ++k) {  // the item's fixed tiles, in order
+        // The item's fixed tiles, in order: this thread's and (MT = 2) the other's. A parity wait tells only two uses
+        // of a slot apart, and the ring's slots change hands (three slots, two tiles an item), so before it leaves the
+        // item the thread has seen the other's tile land too, and a slot is free when both have said so. (With each
+        // waiting for its own alone, a thread could pass the wait for a slot whose last copy, the other's, had not
+        // landed, on the use before that, and release it under the other's MMAs.)
+        int f = 0, other = 0;
+        uint32_t other_ph = 0;
+        for (int k = 0; k < MT; ++k) {
           if (k == m) {
             f = rf.s;
             ok = pf_wait(sm.ffull(f), rf.ph, fail);
+          } else {
+            other = rf.s;
+            other_ph = rf.ph;
           }
           rf.next();
         }
@@ -315,8 +324,10 @@ __device__ __forceinline__ bool pf_pipeline(const PrefillArgs& a, Begin begin, T
             if (ok) umma_commit(sm.sfree(rs.s));
             rs.next();
           }
+        if (ok && MT == 2) ok = pf_wait(sm.ffull(other), other_ph, fail);
         if (!ok) break;
         umma_commit(sm.ffree(f));
+        if (MT == 2) umma_commit(sm.ffree(other));
         ok = items.fetch(sm, fail);
         items.leave(sm);
       }
@@ -338,7 +349,10 @@ __device__ __forceinline__ bool pf_pipeline(const PrefillArgs& a, Begin begin, T
           if (!skip) turn ^= 1u;
           if (!mine) continue;
           if (skip) {
-            if (STATS) {  // releases its share of the normalisers; the copy has landed, so this is the stage's phase
+            // releases its share of the normalisers; the copy has landed, so this is the stage's phase (this set has
+            // seen the stage's last use: the tile it took last is at most three back, as all items of a grid have an
+            // even or all an odd number of tiles)
+            if (STATS) {
               ok = __all_sync(0xffffffffu, pf_wait(sm.full(rs.s), rs.ph, fail));
               if (!ok) break;
               if (lane == 0) mbar_arrive(sm.sdone(rs.s));
