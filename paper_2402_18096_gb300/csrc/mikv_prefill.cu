@@ -19,24 +19,30 @@
 //    tensor cores idle half of the time; the other's MMAs fill its gap. (N = 256 keeps them full from one thread, 1025
 //    clocks for eight MMAs, but then two accumulators fill the tensor memory and all sixteen epilogue warps share
 //    each: 1086 against 1022 us for the whole call below.)
-//  - Two accumulators per fixed tile, so that MMAs run under the arithmetic, and one streamed tile for two fixed ones
-//    (MT = 2), which halves the traffic from L2 per score (the 128-row tiles drew 7.9 TB/s).
-//  - Four sets of four epilogue warps, one set per accumulator, each warp taking whole rows of 128 columns: a hand-over
-//    costs the same whatever the columns behind it. Four warps per scheduler hide each other's tcgen05.ld and
-//    barriers (158 clocks per 32 columns of a warp against 195 with two, 135 for the exponentials alone), so nothing
-//    is prefetched, which keeps the threads within the 96 registers of 19 warps, and one copy of the arithmetic
-//    keeps the loop in the instruction cache.
+//  - Four accumulators, which fill the tensor memory, so that MMAs run under the arithmetic, and one streamed tile for
+//    two fixed ones (MT = 2), which halves the traffic from L2 per score (the 128-row tiles drew 7.9 TB/s).
+//  - Four sets of four epilogue warps. With MT = 2 each has an accumulator of its own, each warp taking whole rows of
+//    128 columns: a hand-over costs the same whatever the columns behind it. Four warps per scheduler hide each other's
+//    tcgen05.ld and barriers (158 clocks per 32 columns of a warp against 195 with two, 135 for the exponentials
+//    alone), so nothing is prefetched, which keeps the threads within the 96 registers of 19 warps, and one copy of the
+//    arithmetic keeps the loop in the instruction cache.
 //  - One persistent CTA per SM whose copies and MMAs run on into the next item (with one item per CTA, filling and
 //    draining cost 9 % of the 4096-token prefill). Items are handed out by the hardware's launch control (a running
 //    CTA takes over the block index of one that has not started), so long and short items balance without a counter
 //    in memory.
+//  - A small prefill has few items (MT = 1) and is bound by the latency of their tiles. There two sets share an
+//    accumulator's columns, four accumulators take turns under one fixed tile and four streamed tiles are in flight,
+//    and at any size pieces of 32 columns that no row of the warp meets are not read. (us of a call with two CTAs per
+//    SM and 64-token streamed tiles / with 8 epilogue warps, two accumulators and three streamed tiles / now: B 1, Hq
+//    32, Hkv 8, T 300: 22.8 / 24.8 / 22.7; B 1, H 32, T 512: 18.4 / 20.5 / 16.6; B 8, H 32, T 300: 35.0 / 37.2 / 33.1;
+//    B 2, H 40, T 777: 42.4 / 49.4 / 37.2.)
 //
-// Where the time goes now (128 x 128 tile and pass, clocks per SM): 1010 of the 512 that exponentials and MMAs each
+// Where the time goes now (128 x 128 tile and pass, clocks per SM): some 950 of the 512 that exponentials and MMAs each
 // need; MMAs with no arithmetic behind them 770, the arithmetic with no MMAs 790 (pass 1) and 930 (pass 2, whose
-// normalisers come from shared memory). B 8, H 32, T 4096: 1211 -> 1022 us; B 1, Hq 32 / Hkv 8, T 32768: 8.59 -> 7.27
+// normalisers come from shared memory). B 8, H 32, T 4096: 1211 -> 965 us; B 1, Hq 32 / Hkv 8, T 32768: 8.59 -> 6.87
 // ms against one CTA per 128-token tile with 64-token streamed tiles, two per SM.
 //
-// The CTA's warps specialise: warps 0 .. 8 MT - 1 take the accumulator rows with tcgen05.ld and do the softmax
+// The CTA's warps specialise: sixteen take the accumulator rows with tcgen05.ld and do the softmax
 // arithmetic; one warp fetches the next item and issues the TMA copies (fixed tiles and a ring of 128B-swizzled
 // streamed tiles, with pass 2's query normalisers), two issue the MMAs. The roles hand tiles over through mbarriers
 // only; every wait is bounded in time and gives up when another role has failed.
@@ -52,35 +58,46 @@ namespace {
 constexpr int kPfTileBytes = kPfTile * kHeadDim * 2;    // 32 KB: 128 tokens x 128 channels, two 64-channel boxes
 constexpr int kPfHalf = kPfTile * 128;                  // one of the boxes
 constexpr int kPfCols = 32;                             // accumulator columns of one tcgen05.ld
-constexpr int kPfStages = 3;                            // streamed tiles in flight
-constexpr int kPfFix = 3;                               // fixed tiles: the current ones and the next item's first
 constexpr int kPfStatBytes = kPfTile * 4;               // pass 2: the streamed queries' log2 normalisers
-constexpr int kPfBars = 3 * kPfStages + 2 * kPfFix + 8 + 4 + 4 + 1;
-constexpr int kPfSmem =
-    1024 + (kPfFix + kPfStages) * kPfTileBytes + kPfStages * kPfStatBytes + 2 * 16 + 8 * kPfBars;
-static_assert(kPfSmem <= 227 * 1024, "shared memory of one SM");
-constexpr int kPfTmemCols = 512;                        // two accumulators of 128 columns per fixed tile
-__host__ __device__ constexpr int pf_threads(int MT) { return 32 * (8 * MT + 3); }  // epilogue, copies, 2 x MMA
+// Six tiles in shared memory: the fixed ones (the current ones and the next item's first) and the streamed ones in
+// flight, of which a small prefill, bound by their latency, wants as many as it can have.
+__host__ __device__ constexpr int pf_fix(int MT) { return MT + 1; }
+__host__ __device__ constexpr int pf_stages(int MT) { return 6 - pf_fix(MT); }
+__host__ __device__ constexpr int pf_bars(int MT) { return 3 * pf_stages(MT) + 2 * pf_fix(MT) + 8 + 4 + 4 + 1; }
+__host__ __device__ constexpr int pf_smem(int MT) {
+  return 1024 + 6 * kPfTileBytes + pf_stages(MT) * kPfStatBytes + 2 * 16 + 8 * pf_bars(MT);
+}
+static_assert(pf_smem(1) <= 227 * 1024 && pf_smem(2) <= 227 * 1024, "shared memory of one SM");
+constexpr int kPfTmemCols = 512;                        // four accumulators of 128 columns
+constexpr int kPfEpi = 16;                              // epilogue warps: four sets of four
+constexpr int kPfThreads = 32 * (kPfEpi + 3);           // epilogue, copies, 2 x MMA
+__host__ __device__ constexpr int pf_accs(int MT) { return 4 / MT; }  // accumulators of a fixed tile
+// Sets that share the columns of an accumulator. With two fixed tiles each of the four accumulators has a set of its
+// own; with one, two sets take the even and two the odd ones.
+__host__ __device__ constexpr int pf_sharers(int MT) { return 2 / MT; }
+__host__ __device__ constexpr int pf_put(int MT) { return 2 * pf_sharers(MT) - 1; }  // sets that hand on their partials
 
+template <int MT>
 struct PfSmem {
+  static constexpr int kStages = pf_stages(MT), kFix = pf_fix(MT);
   uint32_t base;
   __device__ uint32_t fixed(int f) const { return base + f * kPfTileBytes; }
-  __device__ uint32_t stage(int s) const { return base + (kPfFix + s) * kPfTileBytes; }
-  __device__ uint32_t stat(int s) const { return stage(kPfStages) + s * kPfStatBytes; }
-  __device__ uint32_t item(int k) const { return stat(kPfStages) + 16 * k; }
+  __device__ uint32_t stage(int s) const { return base + (kFix + s) * kPfTileBytes; }
+  __device__ uint32_t stat(int s) const { return stage(kStages) + s * kPfStatBytes; }
+  __device__ uint32_t item(int k) const { return stat(kStages) + 16 * k; }
   __device__ uint32_t bar(int i) const { return item(2) + 8 * i; }
   __device__ uint32_t full(int s) const { return bar(s); }                      // copy landed
-  __device__ uint32_t sfree(int s) const { return bar(kPfStages + s); }         // MMAs read it
-  __device__ uint32_t sdone(int s) const { return bar(2 * kPfStages + s); }     // normalisers read
-  __device__ uint32_t ffull(int f) const { return bar(3 * kPfStages + f); }     // fixed tile landed
-  __device__ uint32_t ffree(int f) const { return bar(3 * kPfStages + kPfFix + f); }
-  __device__ uint32_t tfull(int d) const { return bar(3 * kPfStages + 2 * kPfFix + d); }  // accumulator ready
-  __device__ uint32_t tempty(int d) const { return bar(3 * kPfStages + 2 * kPfFix + 4 + d); }  // and read
-  __device__ uint32_t ifull(int k) const { return bar(3 * kPfStages + 2 * kPfFix + 8 + k); }   // next item known
-  __device__ uint32_t iempty(int k) const { return bar(3 * kPfStages + 2 * kPfFix + 10 + k); }
-  __device__ uint32_t pfull(int m) const { return bar(3 * kPfStages + 2 * kPfFix + 12 + m); }  // row partials there
-  __device__ uint32_t pempty(int m) const { return bar(3 * kPfStages + 2 * kPfFix + 14 + m); }  // and taken
-  __device__ uint32_t drain() const { return bar(kPfBars - 1); }
+  __device__ uint32_t sfree(int s) const { return bar(kStages + s); }         // MMAs read it
+  __device__ uint32_t sdone(int s) const { return bar(2 * kStages + s); }     // normalisers read
+  __device__ uint32_t ffull(int f) const { return bar(3 * kStages + f); }     // fixed tile landed
+  __device__ uint32_t ffree(int f) const { return bar(3 * kStages + kFix + f); }
+  __device__ uint32_t tfull(int d) const { return bar(3 * kStages + 2 * kFix + d); }  // accumulator ready
+  __device__ uint32_t tempty(int d) const { return bar(3 * kStages + 2 * kFix + 4 + d); }  // and read
+  __device__ uint32_t ifull(int k) const { return bar(3 * kStages + 2 * kFix + 8 + k); }   // next item known
+  __device__ uint32_t iempty(int k) const { return bar(3 * kStages + 2 * kFix + 10 + k); }
+  __device__ uint32_t pfull(int m) const { return bar(3 * kStages + 2 * kFix + 12 + m); }  // row partials there
+  __device__ uint32_t pempty(int m) const { return bar(3 * kStages + 2 * kFix + 14 + m); }  // and taken
+  __device__ uint32_t drain() const { return bar(pf_bars(MT) - 1); }
 };
 
 // Bounded wait that also gives up as soon as another role of the CTA has failed. The clock is read only every 64
@@ -110,35 +127,46 @@ __device__ __forceinline__ void pf_mma_tile(uint32_t d_tmem, uint32_t fix, uint3
   }
 }
 
-// The work of block index lin. Heads are taken in groups (group_rows / group_cols of them), whole groups one after
-// another: inside a group all heads' longest items come first (so the last items of the grid are short ones), and
-// the group's streamed operand (of the heads that run at the same time) stays within L2.
-// PASS 1: queries q0 .. of query head `head` (b Hq + j), streamed keys 0 .. of its KV head.
+// The work of block index lin. Heads are taken in groups (a.group of them), whole groups one after another: inside a
+// group all heads' longest items come first (so the last items of the grid are short ones), and the group's streamed
+// operand (of the heads that run at the same time) stays within L2.
+// PASS 1: queries q0 .. of query head `head` (b Hq + j), streamed keys 0 .. of its KV head. Pairs of tiles are counted
+// from the last, so that of an odd number the first, whose rows are the shortest, is left alone.
 // PASS 2: keys q0 .. of KV head `head`, streamed queries q0 .. of its G query heads.
 template <int MT, int PASS>
 struct PfWork {
-  int head, q0, heads, n_tiles, str_row, stat_row, m_used;
+  int head, q0, heads, n_tiles, str_row, stat_row, m_used;  // m_used: fixed tiles that are the item's own
 
   __device__ __forceinline__ PfWork(const PrefillArgs& a, int lin) {
     const int G = a.heads_q / a.heads_kv, n_heads = a.batch * (PASS == 1 ? a.heads_q : a.heads_kv);
-    const int items = (a.T + MT * kPfTile - 1) / (MT * kPfTile), per = PASS == 1 ? a.group_rows : a.group_cols;
-    const int grp = lin / (per * items), rem = lin - grp * per * items;
-    const int n = min(per, n_heads - grp * per);  // heads of this group
+    const int tiles = (a.T + kPfTile - 1) / kPfTile, items = (tiles + MT - 1) / MT;
+    const int grp = lin / (a.group * items), rem = lin - grp * a.group * items;
+    const int n = min(a.group, n_heads - grp * a.group);  // heads of this group
     const int it = rem / n;
-    head = grp * per + (rem - it * n);
-    q0 = MT * kPfTile * (PASS == 1 ? items - 1 - it : it);
-    m_used = a.T - q0 > kPfTile ? MT : 1;  // fixed tiles that hold a token
+    head = grp * a.group + (rem - it * n);
+    const int first = PASS == 1 ? tiles - MT * (it + 1) : MT * it;
+    m_used = PASS == 1 ? MT + min(first, 0) : min(MT, tiles - first);
+    q0 = kPfTile * max(first, 0);
     if (PASS == 1) {
       heads = 1;
-      n_tiles = (min(q0 + MT * kPfTile, a.T) + kPfTile - 1) / kPfTile;
+      n_tiles = max(first, 0) + m_used;
       str_row = head / G * a.T;
       stat_row = 0;
     } else {
       heads = G;
-      n_tiles = (a.T - q0 + kPfTile - 1) / kPfTile;
+      n_tiles = tiles - first;
       str_row = head * G * a.T + q0;
       stat_row = head * G * a.T_pad + q0;
     }
+  }
+  // the columns of streamed tile i that rows 32 quarter .. + 31 of fixed tile m meet, in whole pieces of 32: up to the
+  // rows' own tokens (pass 1), from those tokens to the end of the prefill (pass 2); none for rows past the prefill
+  __device__ __forceinline__ int col_begin(int m, int i, int quarter) const {
+    return PASS == 2 && i == m ? 32 * quarter : 0;
+  }
+  __device__ __forceinline__ int col_end(int m, int i, int quarter, int T) const {
+    if (q0 + kPfTile * m + 32 * quarter >= T) return 0;
+    return PASS == 1 ? q0 + kPfTile * (m - i) + 32 * (quarter + 1) : (T - q0 - kPfTile * i + 31) & ~31;
   }
   // tiles wholly on the far side of the diagonal of fixed tile m, and fixed tiles without a token
   __device__ __forceinline__ bool skip(int m, int i) const {
@@ -166,11 +194,13 @@ struct PfItems {
   int lin;
   __device__ __forceinline__ PfItems() : lin((int)blockIdx.x) {}
   // false: no item is left, or a wait failed
-  __device__ __forceinline__ bool fetch(const PfSmem& sm, volatile int* fail) {
+  template <class Smem>
+  __device__ __forceinline__ bool fetch(const Smem& sm, volatile int* fail) {
     if (!pf_wait(sm.ifull(r.s), r.ph, fail)) return false;
     return launch_answer(sm.item(r.s), lin);
   }
-  __device__ __forceinline__ void leave(const PfSmem& sm) {
+  template <class Smem>
+  __device__ __forceinline__ void leave(const Smem& sm) {
     fence_proxy_async_smem();  // our read of the answer precedes the next asynchronous write of the slot
     mbar_arrive(sm.iempty(r.s));
     r.next();
@@ -179,42 +209,45 @@ struct PfItems {
 
 // The pipeline shared by both passes. begin() starts an item on an epilogue thread, tile(w, m, i, col0, v, stat)
 // takes its row of one accumulator (columns col0 .. col0 + 31; stat: shared-memory address of those queries'
-// normalisers, pass 2). Two threads share a row, each taking every other tile: put(row) leaves one's partial result in
-// shared memory, end(w, row) joins it to the other's and closes the row. Returns false when a wait timed out (after draining what
-// was in flight); every role leaves through the final barrier.
+// normalisers, pass 2). Two threads (MT = 1: four) share a row: put(slot) leaves one's partial result in slot k * 128 +
+// row of shared memory (k-th of those that hand theirs on), end(w, row) joins them to its own and closes the row.
+// Returns false when a wait timed out (after draining what was in flight); every role leaves through the final barrier.
 template <int MT, int PASS, class Begin, class Tile, class Put, class End>
 __device__ __forceinline__ bool pf_pipeline(const PrefillArgs& a, Begin begin, Tile tile, Put put, End end) {
   using Work = PfWork<MT, PASS>;
   constexpr bool STATS = PASS == 2;
-  constexpr int kEpi = 8 * MT, kCopyWarp = kEpi, kMmaWarp = kEpi + 1;  // two MMA warps
+  constexpr int kCopyWarp = kPfEpi, kMmaWarp = kPfEpi + 1;  // two MMA warps
+  constexpr int kStages = pf_stages(MT), kFix = pf_fix(MT);
+  constexpr uint32_t kAccs = pf_accs(MT);
+  constexpr int kSharers = pf_sharers(MT), kCols = kPfTile / kSharers;  // a set's columns of an accumulator
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint32_t s_tmem;
   __shared__ int s_fail;
   volatile int* fail = &s_fail;
-  PfSmem sm;
+  PfSmem<MT> sm;
   sm.base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const CUtensorMap* map_fix = PASS == 1 ? &a.map_q : &a.map_k;
   const CUtensorMap* map_str = PASS == 1 ? &a.map_k : &a.map_q;
   if (tid == 0) {
     s_fail = 0;
-    for (int s = 0; s < kPfStages; ++s) {
+    for (int s = 0; s < kStages; ++s) {
       mbar_init(sm.full(s), 1);
       mbar_init(sm.sfree(s), 2);     // both MMA threads
-      mbar_init(sm.sdone(s), 4 * MT);  // the warps whose turn the tile is
+      mbar_init(sm.sdone(s), kPfEpi / 2);  // the warps whose turn the tile is
     }
-    for (int f = 0; f < kPfFix; ++f) {
+    for (int f = 0; f < kFix; ++f) {
       mbar_init(sm.ffull(f), 1);
       mbar_init(sm.ffree(f), 2);     // both MMA threads
     }
     for (int d = 0; d < 4; ++d) {
       mbar_init(sm.tfull(d), 1);
-      mbar_init(sm.tempty(d), 4);
+      mbar_init(sm.tempty(d), 4 * kSharers);
     }
     for (int k = 0; k < 2; ++k) {
       mbar_init(sm.ifull(k), 1);
-      mbar_init(sm.iempty(k), kEpi + 2);  // the epilogue warps and the MMA threads
-      mbar_init(sm.pfull(k), 4);
+      mbar_init(sm.iempty(k), kPfEpi + 2);  // the epilogue warps and the MMA threads
+      mbar_init(sm.pfull(k), 4 * pf_put(MT));
       mbar_init(sm.pempty(k), 4);
     }
     mbar_init(sm.drain(), 2);
@@ -231,8 +264,8 @@ __device__ __forceinline__ bool pf_pipeline(const PrefillArgs& a, Begin begin, T
   const uint32_t tmem = s_tmem;
 
   // the copy thread's record of what it has in flight (drained if a wait fails)
-  PfRing<kPfStages> rs;
-  PfRing<kPfFix> rf;
+  PfRing<kStages> rs;
+  PfRing<kFix> rf;
   int n_str = 0, n_fix = 0;
   bool asked = false;
   PfItems items;
@@ -253,7 +286,7 @@ __device__ __forceinline__ bool pf_pipeline(const PrefillArgs& a, Begin begin, T
             if (m < MT) {  // the item's fixed tiles go between its first streamed ones (both even if one is unused)
               const int last = w.heads * w.n_tiles == 1 ? MT : m + 1;
               for (; m < last && ok; ++m) {
-                if (n_fix >= kPfFix && !(ok = pf_wait(sm.ffree(rf.s), rf.ph ^ 1u, fail))) break;
+                if (n_fix >= kFix && !(ok = pf_wait(sm.ffree(rf.s), rf.ph ^ 1u, fail))) break;
                 ++n_fix;
                 mbar_arrive_expect_tx(sm.ffull(rf.s), kPfTileBytes);
                 tma_load_2d(sm.fixed(rf.s), map_fix, 0, fix_row + kPfTile * m, sm.ffull(rf.s));
@@ -262,7 +295,7 @@ __device__ __forceinline__ bool pf_pipeline(const PrefillArgs& a, Begin begin, T
               }
               if (!ok) break;
             }
-            if (n_str >= kPfStages)
+            if (n_str >= kStages)
               ok = pf_wait(sm.sfree(rs.s), rs.ph ^ 1u, fail) && (!STATS || pf_wait(sm.sdone(rs.s), rs.ph ^ 1u, fail));
             if (!ok) break;
             ++n_str;
@@ -286,7 +319,7 @@ __device__ __forceinline__ bool pf_pipeline(const PrefillArgs& a, Begin begin, T
     if (lane == 0) {  // MMAs: a tile into a free accumulator once its copy landed
       // MT = 2: the thread multiplies fixed tile p with every streamed tile; MT = 1: the two take turns
       const int p = warp - kMmaWarp, m = MT == 2 ? p : 0;
-      uint32_t uses = 0;  // accumulator uses of fixed tile m: buffer bit 0, parity bit 1
+      uint32_t uses = 0;  // accumulator uses of fixed tile m: buffer in the low bits, parity above
       bool ok = true;
       while (ok) {
         const Work w(a, items.lin);
@@ -311,9 +344,9 @@ __device__ __forceinline__ bool pf_pipeline(const PrefillArgs& a, Begin begin, T
           for (int i = 0; i < w.n_tiles && ok; ++i) {
             ok = pf_wait(sm.full(rs.s), rs.ph, fail);
             if (ok && !w.skip(m, i)) {
-              const int d = 2 * m + (int)(uses & 1u);
+              const int d = kAccs * m + (int)(uses % kAccs);
               if (MT == 2 || (int)(uses & 1u) == p) {
-                ok = pf_wait(sm.tempty(d), ((uses >> 1) & 1u) ^ 1u, fail);
+                ok = pf_wait(sm.tempty(d), ((uses / kAccs) & 1u) ^ 1u, fail);
                 if (!ok) break;
                 tcgen05_after_sync();
                 pf_mma_tile(tmem + (uint32_t)(d * kPfTile), sm.fixed(f), sm.stage(rs.s));
@@ -334,11 +367,14 @@ __device__ __forceinline__ bool pf_pipeline(const PrefillArgs& a, Begin begin, T
       umma_commit(sm.drain());  // every MMA issued has completed once both arrive
       if (!mbar_wait(sm.drain(), 0)) record_error(a.status, kErrDrainTimeout);
     }
-  } else {  // epilogue warps: fixed tile m, every other of its accumulators (d = 2 m + p), lanes 32 (w % 4) ..
-    const int m = warp >> 3, p = (warp >> 2) & 1, d = 2 * m + p;
-    const uint32_t acc = tmem + (uint32_t)(d * kPfTile) + ((uint32_t)(32 * (warp & 3)) << 16);
+  } else {  // epilogue warps: fixed tile m, every other of its accumulators (from the p-th), lanes 32 (w % 4) ..,
+            // columns first .. first + kCols - 1
+    const int set = warp >> 2, p = set & 1, m = MT == 2 ? set >> 1 : 0;
+    const int first = MT == 2 ? 0 : kCols * (set >> 1);
+    const uint32_t lanes = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
     const int row = kPfTile * m + 32 * (warp & 3) + lane;
-    uint32_t turn = 0, use = 0, closed = 0;  // whose turn; parities of this accumulator's uses and of the items
+    const int part = MT == 2 ? p : set;  // 0: closes the rows
+    uint32_t turn = 0, uses = 0, closed = 0;  // whose turn; accumulators taken; parity of the items
     bool ok = true;
     while (ok) {
       const Work w(a, items.lin);
@@ -359,18 +395,22 @@ __device__ __forceinline__ bool pf_pipeline(const PrefillArgs& a, Begin begin, T
             }
             continue;
           }
-          ok = __all_sync(0xffffffffu, pf_wait(sm.tfull(d), use, fail));
+          const int d = (int)kAccs * m + p + 2 * (int)(uses % (kAccs / 2));
+          ok = __all_sync(0xffffffffu, pf_wait(sm.tfull(d), (uses / (kAccs / 2)) & 1u, fail));
           // the staged normalisers: observe their copy's completion directly (it has completed: the MMAs
           // that produced this accumulator waited for it, and the stage is not refilled before sdone)
           if (STATS && ok) ok = __all_sync(0xffffffffu, pf_wait(sm.full(rs.s), rs.ph, fail));
           if (!ok) break;
-          use ^= 1u;
+          ++uses;
           tcgen05_after_sync();
+          const int c1 = min(first + kCols, w.col_end(m, i, warp & 3, a.T));
+          int c = max(first, w.col_begin(m, i, warp & 3));
+          if (c >= c1 && lane == 0) mbar_arrive(sm.tempty(d));  // (nothing to read)
 #pragma unroll 1  // (one copy of the arithmetic: the instruction cache was a limit)
-          for (int c = 0; c < kPfTile; c += kPfCols) {
+          for (; c < c1; c += kPfCols) {
             float v[kPfCols];
-            tmem_ld32(acc + c, v);
-            if (c == kPfTile - kPfCols) {  // the accumulator has been read
+            tmem_ld32(lanes + (uint32_t)(d * kPfTile + c), v);
+            if (c + kPfCols >= c1) {  // this warp's share of the accumulator has been read
               tcgen05_before_sync();
               __syncwarp();
               if (lane == 0) mbar_arrive(sm.tempty(d));
@@ -381,11 +421,11 @@ __device__ __forceinline__ bool pf_pipeline(const PrefillArgs& a, Begin begin, T
           if (STATS && lane == 0) mbar_arrive(sm.sdone(rs.s));
         }
       if (!ok) break;
-      if (m < w.m_used) {  // the warps of the second accumulator hand their rows' partials to those of the first
-        if (p != 0) {
+      if (m < w.m_used) {  // the other sets of the fixed tile hand their rows' partials to its first
+        if (part != 0) {
           ok = __all_sync(0xffffffffu, pf_wait(sm.pempty(m), closed ^ 1u, fail));
           if (!ok) break;
-          put(row);
+          put(kPfTile * (part - 1) + row);
           __syncwarp();
           if (lane == 0) mbar_arrive(sm.pfull(m));
         } else {
@@ -411,14 +451,14 @@ __device__ __forceinline__ bool pf_pipeline(const PrefillArgs& a, Begin begin, T
   if (failed) {
     if (tid == 0) record_error(a.status, kErrFullTimeout);
     if (warp == kCopyWarp && lane == 0) {  // no copy may outlive the CTA
-      for (int v = 0; v < min(n_str, kPfStages); ++v) {  // the last uses of the ring, latest first
+      for (int v = 0; v < min(n_str, kStages); ++v) {  // the last uses of the ring, latest first
         rs.ph ^= rs.s == 0 ? 1u : 0u;
-        rs.s = rs.s == 0 ? kPfStages - 1 : rs.s - 1;
+        rs.s = rs.s == 0 ? kStages - 1 : rs.s - 1;
         if (!mbar_wait(sm.full(rs.s), rs.ph)) record_error(a.status, kErrDrainTimeout);
       }
-      for (int v = 0; v < min(n_fix, kPfFix); ++v) {
+      for (int v = 0; v < min(n_fix, kFix); ++v) {
         rf.ph ^= rf.s == 0 ? 1u : 0u;
-        rf.s = rf.s == 0 ? kPfFix - 1 : rf.s - 1;
+        rf.s = rf.s == 0 ? kFix - 1 : rf.s - 1;
         if (!mbar_wait(sm.ffull(rf.s), rf.ph)) record_error(a.status, kErrDrainTimeout);
       }
       if (asked && !mbar_wait(sm.ifull(items.r.s), items.r.ph)) record_error(a.status, kErrDrainTimeout);
@@ -461,6 +501,15 @@ __device__ __forceinline__ float pf_exp_sum(const float (&v)[kPfCols], float sca
   return pf_sum8(acc);
 }
 
+// A row's sum from its closing thread's and those handed on. Which of two accumulators an item begins with depends on
+// the items its block had before, so the two that share columns are added first: their sum is the same either way.
+template <int MT, class Part>
+__device__ __forceinline__ float pf_join(float own, Part part) {
+  const float sum = own + part(0);
+  if constexpr (MT == 2) return sum;
+  else return sum + (part(1) + part(2));
+}
+
 // ------------------------------------------------------------------------------- pass 1: row statistics
 //
 // Per query row the softmax normaliser is accumulated against a reference r (log2 units): the exact maximum
@@ -469,10 +518,10 @@ __device__ __forceinline__ float pf_exp_sum(const float (&v)[kPfCols], float sca
 // normaliser as the true maximum; the kernel stores its log2, r + log2(sum), negated (pass 2 adds it).
 
 template <int MT>
-__global__ void __launch_bounds__(pf_threads(MT), 1) prefill_rows_kernel(const __grid_constant__ PrefillArgs a) {
+__global__ void __launch_bounds__(kPfThreads, 1) prefill_rows_kernel(const __grid_constant__ PrefillArgs a) {
   using Work = PfWork<MT, 1>;
-  __shared__ float s_r[MT * kPfTile], s_l[MT * kPfTile];  // one thread's partial of each row
-  float r = -INFINITY, l = 0.f;                           // over this thread's tiles
+  __shared__ float s_r[MT * pf_put(MT) * kPfTile], s_l[MT * pf_put(MT) * kPfTile];  // the partials handed on
+  float r = -INFINITY, l = 0.f;  // over this thread's tiles and columns
   pf_pipeline<MT, 1>(
       a,
       [&] {
@@ -498,15 +547,19 @@ __global__ void __launch_bounds__(pf_threads(MT), 1) prefill_rows_kernel(const _
         }
         l += sum;
       },
-      [&](int row) {
-        s_r[row] = r;
-        s_l[row] = l;
+      [&](int slot) {
+        s_r[slot] = r;
+        s_l[slot] = l;
       },
-      [&](const Work& w, int row) {  // both partials against the larger reference
+      [&](const Work& w, int row) {  // the partials against the largest reference
         const int q = w.q0 + row;
-        const float r2 = s_r[row], rm = fmaxf(r, r2);
-        const float lt = (r == -INFINITY ? 0.f : l * fast_exp2(r - rm)) +
-                         (r2 == -INFINITY ? 0.f : s_l[row] * fast_exp2(r2 - rm));
+        float rm = r;
+#pragma unroll
+        for (int k = 0; k < pf_put(MT); ++k) rm = fmaxf(rm, s_r[kPfTile * k + row]);
+        const float lt = pf_join<MT>(r == -INFINITY ? 0.f : l * fast_exp2(r - rm), [&](int k) {
+          const float r2 = s_r[kPfTile * k + row];
+          return r2 == -INFINITY ? 0.f : s_l[kPfTile * k + row] * fast_exp2(r2 - rm);
+        });
         a.stats[(size_t)w.head * a.T_pad + q] = q < a.T ? -(rm + log2f(lt)) : -INFINITY;
       });
 }
@@ -514,9 +567,9 @@ __global__ void __launch_bounds__(pf_threads(MT), 1) prefill_rows_kernel(const _
 // ------------------------------------------------------------------------------ pass 2: column sums
 
 template <int MT>
-__global__ void __launch_bounds__(pf_threads(MT), 1) prefill_cols_kernel(const __grid_constant__ PrefillArgs a) {
+__global__ void __launch_bounds__(kPfThreads, 1) prefill_cols_kernel(const __grid_constant__ PrefillArgs a) {
   using Work = PfWork<MT, 2>;
-  __shared__ float s_cs[MT * kPfTile];  // one thread's sum of each row
+  __shared__ float s_cs[MT * pf_put(MT) * kPfTile];  // the sums handed on
   float cs = 0.f;
   pf_pipeline<MT, 2>(
       a, [&] { cs = 0.f; },
@@ -545,41 +598,49 @@ __global__ void __launch_bounds__(pf_threads(MT), 1) prefill_cols_kernel(const _
         }
         cs += pf_sum8(acc);
       },
-      [&](int row) { s_cs[row] = cs; },
+      [&](int slot) { s_cs[slot] = cs; },
       [&](const Work& w, int row) {
-        if (w.q0 + row < a.T) a.scores[(size_t)w.head * a.T + w.q0 + row] = cs + s_cs[row];
+        const float sum = pf_join<MT>(cs, [&](int k) { return s_cs[kPfTile * k + row]; });
+        if (w.q0 + row < a.T) a.scores[(size_t)w.head * a.T + w.q0 + row] = sum;
       });
 }
 
-template <int MT>
-cudaError_t pf_launch(PrefillArgs a, cudaStream_t st) {
+template <class Kernel>
+cudaError_t pf_launch(Kernel kernel, int smem, PrefillArgs a, int items, int n_heads, cudaStream_t st) {
+  const int per = (2 * kPfSlots + items - 1) / items;  // heads per group: about two rounds of the resident CTAs,
+  const int groups = max(1, n_heads / per);            // in groups of like size: the long items of a small last group
+  a.group = (n_heads + groups - 1) / groups;           // ran alone at the end (80 heads as 76 and 4, T 777: 46 / 37 us)
+  kernel<<<items * n_heads, kPfThreads, smem, st>>>(a);
+  return cudaGetLastError();
+}
+
+// One pass with items of two fixed tiles when there are then at least three for two SMs, else of one, which gives a
+// small prefill twice the CTAs. us of a pass, one tile against two, by the items of two: rows, 96: 9.9 / 10.7, 160: 13.2
+// / 14.5, 192: 17.2 / 20.2, 256: 23.5 / 26.4 and 13.7 / 11.7, 384: 17.6 / 15.5; columns, 72: 61.9 / 100.7, 152: 131.6 /
+// 150.9, 192: 17.9 / 22.0, 256: 17.6 / 19.0 and 13.5 / 11.9, 384: 48.6 / 44.8, 512: 589 / 486.
+template <int PASS>
+cudaError_t pf_pass(const PrefillArgs& a, cudaStream_t st) {
+  constexpr auto one = PASS == 1 ? prefill_rows_kernel<1> : prefill_cols_kernel<1>;
+  constexpr auto two = PASS == 1 ? prefill_rows_kernel<2> : prefill_cols_kernel<2>;
   static bool configured = false;
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(prefill_rows_kernel<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPfSmem);
+    cudaError_t e = cudaFuncSetAttribute(one, cudaFuncAttributeMaxDynamicSharedMemorySize, pf_smem(1));
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(prefill_cols_kernel<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPfSmem);
+    e = cudaFuncSetAttribute(two, cudaFuncAttributeMaxDynamicSharedMemorySize, pf_smem(2));
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  const int items = (a.T + MT * kPfTile - 1) / (MT * kPfTile);
-  const int per = (2 * kPfSlots + items - 1) / items;  // heads per group: about two rounds of the resident CTAs
-  a.group_rows = a.group_cols = per;
-  prefill_rows_kernel<MT><<<items * a.batch * a.heads_q, pf_threads(MT), kPfSmem, st>>>(a);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  prefill_cols_kernel<MT><<<items * a.batch * a.heads_kv, pf_threads(MT), kPfSmem, st>>>(a);
-  return cudaGetLastError();
+  const int tiles = (a.T + kPfTile - 1) / kPfTile, n_heads = a.batch * (PASS == 1 ? a.heads_q : a.heads_kv);
+  const int items2 = (tiles + 1) / 2;
+  return 2ll * items2 * n_heads >= 3ll * kPfSlots ? pf_launch(two, pf_smem(2), a, items2, n_heads, st)
+                                                  : pf_launch(one, pf_smem(1), a, tiles, n_heads, st);
 }
 
 }  // namespace
 
-// Items of two fixed tiles when pass 2 then still has one per SM (its items are the fewer ones), else of one, which
-// gives a small prefill twice the CTAs. Either side measured, one tile against two: Hkv 8, T 4864 (152 items of two
-// tiles) 280.9 / 248.5 us, T 3000 (96) 151.1 / 155.0 us, T 2048 (64) 84.5 / 99.9 us, T 8192 (256) 749 / 599 us;
-// H 32, T 608, B 2 (192) 32.8 / 29.2 us, T 512, B 1 (64) 20.6 / 21.0 us.
 cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st) {
-  const int items2 = (a.T + 2 * kPfTile - 1) / (2 * kPfTile);
-  return (long long)items2 * a.batch * a.heads_kv >= kPfSlots ? pf_launch<2>(a, st) : pf_launch<1>(a, st);
+  const cudaError_t e = pf_pass<1>(a, st);
+  return e != cudaSuccess ? e : pf_pass<2>(a, st);
 }
 
 }  // namespace mikv

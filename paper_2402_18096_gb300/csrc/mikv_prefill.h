@@ -22,7 +22,7 @@ struct PrefillArgs {
   float* scores;      // [B * Hkv][T]
   int* status;        // workspace status word
   int batch, heads_q, heads_kv, T, T_pad;  // T_pad = T rounded up to a whole tile
-  int group_rows, group_cols;  // heads taken together by the two passes' block order
+  int group;          // heads taken together by a pass's block order
   float scale_log2;   // sm_scale * log2(e)
 };
 
