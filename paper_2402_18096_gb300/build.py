@@ -26,6 +26,8 @@ SOURCES = ["mikv_attn_h16.cu", "mikv_attn_h8.cu", "mikv_attn_h4.cu", "mikv_attn_
 PYCALL = "mikv_pycall.c"  # the binding's decode-path calls as an extension module (where Python's headers are installed)
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
+# a register spilled in the kernels that load from tensor memory is an error (see tmem_ld32)
+SOURCE_FLAGS = {"mikv_prefill.cu": ["-Xptxas", "-warn-spills,-Werror"]}
 
 
 def _nvcc() -> str:
@@ -33,6 +35,10 @@ def _nvcc() -> str:
         if cand and os.path.exists(cand):
             return cand
     raise RuntimeError("nvcc not found: the CUDA toolkit is required to build libmikv")
+
+
+def source_flags(src: str, debug: bool = False) -> list:
+    return NVCC_FLAGS + SOURCE_FLAGS.get(src, []) + (["-DMIKV_DEBUG"] if debug else [])
 
 
 def _inputs():
@@ -77,11 +83,10 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
         return lib
     os.makedirs(out_dir, exist_ok=True)
     nvcc = _nvcc()
-    flags = NVCC_FLAGS + (["-DMIKV_DEBUG"] if debug else [])
 
     def compile_one(src):
         obj = os.path.join(out_dir, os.path.splitext(src)[0] + ".o")
-        cmd = [nvcc, *ARCH, *flags, "-c", os.path.join(CSRC, src), "-o", obj]
+        cmd = [nvcc, *ARCH, *source_flags(src, debug), "-c", os.path.join(CSRC, src), "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed on {src}:\n{r.stdout}\n{r.stderr}")

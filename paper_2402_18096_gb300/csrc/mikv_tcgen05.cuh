@@ -58,9 +58,9 @@ __device__ __forceinline__ void tcgen05_before_sync() { asm volatile("tcgen05.fe
 __device__ __forceinline__ void tcgen05_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 // 32 consecutive fp32 columns of this thread's TMEM lane (warp w reads lanes 32 (w % 4) ..), loaded and waited for in
-// one statement. With the wait in a statement of its own, a register copy can sit between the two and keep the value
-// from before the load: kernels written so gave sums that changed from run to run (12 of 72 passes over 32768 tokens),
-// and so did one that spilled a register here. A kernel that uses it must compile without spills (-Xptxas -v).
+// one statement, so that no register copy can be put between the two. A kernel that uses it must compile without spills:
+// the build makes one an error (a variant that spilled a register by the load gave sums that changed from run to run;
+// why is not known).
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n\t"
                "tcgen05.wait::ld.sync.aligned;"
