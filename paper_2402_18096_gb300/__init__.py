@@ -14,6 +14,7 @@ import importlib.util
 import math
 import os
 import threading
+import warnings
 from dataclasses import dataclass
 
 import torch
@@ -63,6 +64,22 @@ _pycall = None  # mikv_pycall, the decode-path calls in C (None: not built here,
 _lock = threading.Lock()
 
 
+def _load_pycall(path, lib):
+    """The extension module bound to lib, or None when it is not built or this interpreter cannot load it."""
+    if not os.path.exists(path):
+        return None
+    try:
+        loader = importlib.machinery.ExtensionFileLoader("mikv_pycall", path)
+        mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("mikv_pycall", loader))
+        loader.exec_module(mod)
+    except ImportError as e:
+        warnings.warn(f"{path} cannot be loaded, the decode calls go through ctypes: {e}")
+        return None
+    mod.bind(*[ctypes.cast(getattr(lib, f), ctypes.c_void_p).value for f in ("mikv_decode_step", "mikv_decode_attention")],
+             torch.float32)
+    return mod
+
+
 def load(build_if_missing: bool = True) -> ctypes.CDLL:
     """Load libmikv.so (building it with nvcc first when it is missing or stale). With MIKV_DEBUG=1 in the
     environment the checked build (libmikv_debug.so, -DMIKV_DEBUG) is loaded instead."""
@@ -104,14 +121,7 @@ def load(build_if_missing: bool = True) -> ctypes.CDLL:
             for name, (res, args) in sig.items():
                 fn = getattr(lib, name)
                 fn.restype, fn.argtypes = res, args
-            pycall = _build.pycall_path(debug)
-            if os.path.exists(pycall):
-                loader = importlib.machinery.ExtensionFileLoader("mikv_pycall", pycall)
-                mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("mikv_pycall", loader))
-                loader.exec_module(mod)
-                mod.bind(*[ctypes.cast(getattr(lib, f), P).value for f in ("mikv_decode_step", "mikv_decode_attention")],
-                         torch.float32)
-                _pycall = mod
+            _pycall = _load_pycall(_build.pycall_path(debug), lib)
             _lib = lib
     return _lib
 

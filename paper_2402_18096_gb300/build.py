@@ -12,10 +12,12 @@ import shutil
 import subprocess
 import sys
 import sysconfig
+import warnings
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
+HEADER = os.path.join(os.path.dirname(HERE), "include", "mikv.h")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libmikv.so")
 OUT_DIR_DEBUG = os.path.join(HERE, "_build_debug")
@@ -43,45 +45,61 @@ def source_flags(src: str, debug: bool = False) -> list:
 
 def _inputs():
     files = [os.path.join(CSRC, s) for s in SOURCES]
-    files += [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h", ".c"))]
-    files.append(os.path.join(os.path.dirname(HERE), "include", "mikv.h"))
-    return files
+    files += [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
+    return files + [HEADER]
 
 
 def pycall_path(debug: bool = False) -> str:
-    return os.path.join(OUT_DIR_DEBUG if debug else OUT_DIR, "mikv_pycall.so")
+    """The extension module of this interpreter (its ABI is part of the name: another one builds its own)."""
+    return os.path.join(OUT_DIR_DEBUG if debug else OUT_DIR, "mikv_pycall" + sysconfig.get_config_var("EXT_SUFFIX"))
+
+
+def _pycall_tools():
+    """(C compiler, folder of Python's headers), or None where one is missing."""
+    include = sysconfig.get_paths()["include"]
+    cc = shutil.which("gcc") or shutil.which("cc")
+    return (cc, include) if cc and os.path.exists(os.path.join(include, "Python.h")) else None
 
 
 def _build_pycall(debug: bool) -> None:
-    """The extension module, or none (and no stale one) without Python's headers or a C compiler."""
-    out = pycall_path(debug)
-    include = sysconfig.get_paths()["include"]
-    gcc = shutil.which("gcc") or shutil.which("cc")
-    if not gcc or not os.path.exists(os.path.join(include, "Python.h")):
-        if os.path.exists(out):
-            os.unlink(out)
-        return
-    tmp = out + f".tmp{os.getpid()}"
-    cmd = [gcc, "-O2", "-std=c11", "-shared", "-fPIC", "-Wall", "-I", include, os.path.join(CSRC, PYCALL), "-o", tmp]
-    r = subprocess.run(cmd, capture_output=True, text=True)
-    if r.returncode != 0:
-        raise RuntimeError(f"{gcc} failed on {PYCALL}:\n{r.stdout}\n{r.stderr}")
-    os.replace(tmp, out)
+    """The optional extension module: without the tools, or if it does not compile, there is none (and no stale one), and
+    the calls go through ctypes."""
+    out, tools = pycall_path(debug), _pycall_tools()
+    if tools:
+        tmp = out + f".tmp{os.getpid()}"
+        cmd = [tools[0], "-O2", "-std=c11", "-shared", "-fPIC", "-Wall", "-I", tools[1], os.path.join(CSRC, PYCALL), "-o", tmp]
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        if r.returncode == 0:
+            os.replace(tmp, out)
+            return
+        warnings.warn(f"{tools[0]} failed on {PYCALL}, the decode calls go through ctypes:\n{r.stdout}\n{r.stderr}")
+    if os.path.exists(out):
+        os.unlink(out)
+
+
+def _current(target: str, inputs) -> bool:
+    return os.path.exists(target) and all(os.path.getmtime(f) <= os.path.getmtime(target) for f in inputs)
+
+
+def _lib_current(debug: bool) -> bool:
+    return _current(LIB_DEBUG if debug else LIB, _inputs())
+
+
+def _pycall_current(debug: bool) -> bool:
+    return not _pycall_tools() or _current(pycall_path(debug), [os.path.join(CSRC, PYCALL), HEADER])
 
 
 def up_to_date(debug: bool = False) -> bool:
-    lib = LIB_DEBUG if debug else LIB
-    if not os.path.exists(lib):
-        return False
-    t = os.path.getmtime(lib)
-    return all(os.path.getmtime(f) <= t for f in _inputs())
+    return _lib_current(debug) and _pycall_current(debug)
 
 
 def build(force: bool = False, verbose: bool = False, debug: bool = False) -> str:
     lib, out_dir = (LIB_DEBUG, OUT_DIR_DEBUG) if debug else (LIB, OUT_DIR)
-    if not force and up_to_date(debug):
-        return lib
     os.makedirs(out_dir, exist_ok=True)
+    if force or not _pycall_current(debug):
+        _build_pycall(debug)
+    if not force and _lib_current(debug):
+        return lib
     nvcc = _nvcc()
 
     def compile_one(src):
@@ -94,7 +112,6 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
             print(r.stdout, r.stderr, file=sys.stderr)
         return obj
 
-    _build_pycall(debug)
     with ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
         objs = list(ex.map(compile_one, SOURCES))
     tmp = lib + f".tmp{os.getpid()}"

@@ -1,8 +1,11 @@
-"""The build: what it refuses."""
+"""The build: what it refuses, and the optional extension module beside the library."""
+import os
 import subprocess
+import sysconfig
 
 import pytest
 
+import paper_2402_18096_gb300 as pkg
 from paper_2402_18096_gb300 import build as libbuild
 
 SOURCE = """
@@ -36,8 +39,64 @@ def test_spill_by_a_tensor_memory_load_is_an_error(tmp_path, debug):
 
 
 def test_users_of_tensor_memory_loads_are_covered():
-    import os
     for name in libbuild.SOURCES:
         with open(os.path.join(libbuild.CSRC, name)) as f:
             if "tmem_ld32" in f.read():
                 assert name in libbuild.SOURCE_FLAGS
+
+
+needs_tools = pytest.mark.skipif(libbuild._pycall_tools() is None, reason="no C compiler or no Python headers")
+
+
+@pytest.fixture
+def out_dir(tmp_path, monkeypatch):
+    """An output folder whose library is current and which holds no extension module."""
+    monkeypatch.setattr(libbuild, "OUT_DIR", str(tmp_path))
+    monkeypatch.setattr(libbuild, "LIB", str(tmp_path / "libmikv.so"))
+    (tmp_path / "libmikv.so").write_bytes(b"")
+    return tmp_path
+
+
+@needs_tools
+def test_module_is_built_when_missing_or_stale(out_dir):
+    """The module carries this interpreter's ABI in its name, and the library being current does not hide its absence or
+    its age. The library is not built again for it."""
+    module = libbuild.pycall_path()
+    assert module.endswith(sysconfig.get_config_var("EXT_SUFFIX")) and os.path.dirname(module) == str(out_dir)
+    assert not libbuild.up_to_date()
+    libbuild.build()
+    assert os.path.getsize(module) > 0 and libbuild.up_to_date()
+    os.utime(module, (1, 1))
+    assert not libbuild.up_to_date()
+    libbuild.build()
+    assert libbuild.up_to_date() and (out_dir / "libmikv.so").read_bytes() == b""
+
+
+@needs_tools
+def test_module_that_does_not_compile_is_left_out(out_dir, monkeypatch):
+    """A failing compiler costs the module, not the library, and leaves no older module behind."""
+    module = libbuild.pycall_path()
+    with open(module, "wb"):
+        os.utime(module, (1, 1))
+    bad = out_dir / "cc"
+    bad.write_text("#!/bin/sh\necho no such header; exit 1\n")
+    bad.chmod(0o755)
+    monkeypatch.setattr(libbuild, "_pycall_tools", lambda: (str(bad), "/nowhere"))
+    with pytest.warns(UserWarning, match="ctypes"):
+        assert libbuild.build() == str(out_dir / "libmikv.so")
+    assert not os.path.exists(module)
+
+
+def test_module_that_does_not_load_is_left_out(tmp_path):
+    lib = pkg.load()
+    bad = tmp_path / "mikv_pycall.so"
+    bad.write_bytes(b"not a shared object")
+    with pytest.warns(UserWarning, match="ctypes"):
+        assert pkg._load_pycall(str(bad), lib) is None
+    assert pkg._load_pycall(str(tmp_path / "none.so"), lib) is None
+
+
+@needs_tools
+def test_module_is_loaded_where_it_can_be_built():
+    pkg.load()
+    assert pkg._pycall is not None
