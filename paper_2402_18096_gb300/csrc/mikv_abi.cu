@@ -391,7 +391,7 @@ mikv_status mikv_quantize_pack(const mikv_shape* shape, const mikv_cache* cache,
                                          static_cast<cudaStream_t>(stream)));
   }
   return cuda_status(launch_quantize_pack(*shape, *cache, k_src, v_src, src_tok, n_src, rows, n_rows, lo_start,
-                                          static_cast<cudaStream_t>(stream)));
+                                          num_sms(), static_cast<cudaStream_t>(stream)));
 }
 
 mikv_status mikv_prefill_scores(const mikv_shape* shape, const void* q_pre, const void* k_pre, int32_t T,
@@ -425,7 +425,7 @@ mikv_status mikv_prefill_scores(const mikv_shape* shape, const void* q_pre, cons
   a.T = T;
   a.T_pad = prefill_padded(T);
   a.scale_log2 = sm_scale * 1.4426950408889634f;
-  return cuda_status(launch_prefill(a, static_cast<cudaStream_t>(stream)));
+  return cuda_status(launch_prefill(a, num_sms(), static_cast<cudaStream_t>(stream)));
 }
 
 mikv_status mikv_decode_attention(const mikv_shape* shape, const mikv_cache* cache, int32_t n_lo, const void* q,

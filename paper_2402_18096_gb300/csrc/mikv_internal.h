@@ -191,7 +191,7 @@ cudaError_t launch_merge(const MergeArgs& a, int G, int out_f32, cudaStream_t st
 
 cudaError_t launch_quantize_pack(const mikv_shape& s, const mikv_cache& c, const void* k_src,
                                  const void* v_src, const int32_t* src_tok, int n_src,
-                                 const int32_t* rows, int n_rows, int lo_start, cudaStream_t st);
+                                 const int32_t* rows, int n_rows, int lo_start, int num_sms, cudaStream_t st);
 
 // Per-channel retained keys (App. C): append rows at retained positions p0 .. p0 + n_rows - 1 (quantizing
 // every group of 64 that completes, staging the rest in important rows hi_cap ..); with n_rows == 0 and

@@ -606,10 +606,10 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_cols_kernel(const __gri
 }
 
 template <class Kernel>
-cudaError_t pf_launch(Kernel kernel, int smem, PrefillArgs a, int items, int n_heads, cudaStream_t st) {
-  const int per = (2 * kPfSlots + items - 1) / items;  // heads per group: about two rounds of the resident CTAs,
-  const int groups = max(1, n_heads / per);            // in groups of like size: the long items of a small last group
-  a.group = (n_heads + groups - 1) / groups;           // ran alone at the end (80 heads as 76 and 4, T 777: 46 / 37 us)
+cudaError_t pf_launch(Kernel kernel, int smem, PrefillArgs a, int items, int n_heads, int num_sms, cudaStream_t st) {
+  const int per = (2 * num_sms + items - 1) / items;  // heads per group: about two rounds of the resident CTAs,
+  const int groups = max(1, n_heads / per);           // in groups of like size: the long items of a small last group
+  a.group = (n_heads + groups - 1) / groups;          // ran alone at the end (80 heads as 76 and 4, T 777: 46 / 37 us)
   kernel<<<items * n_heads, kPfThreads, smem, st>>>(a);
   return cudaGetLastError();
 }
@@ -619,7 +619,7 @@ cudaError_t pf_launch(Kernel kernel, int smem, PrefillArgs a, int items, int n_h
 // / 14.5, 192: 17.2 / 20.2, 256: 23.5 / 26.4 and 13.7 / 11.7, 384: 17.6 / 15.5; columns, 72: 61.9 / 100.7, 152: 131.6 /
 // 150.9, 192: 17.9 / 22.0, 256: 17.6 / 19.0 and 13.5 / 11.9, 384: 48.6 / 44.8, 512: 589 / 486.
 template <int PASS>
-cudaError_t pf_pass(const PrefillArgs& a, cudaStream_t st) {
+cudaError_t pf_pass(const PrefillArgs& a, int num_sms, cudaStream_t st) {
   constexpr auto one = PASS == 1 ? prefill_rows_kernel<1> : prefill_cols_kernel<1>;
   constexpr auto two = PASS == 1 ? prefill_rows_kernel<2> : prefill_cols_kernel<2>;
   static bool configured = false;
@@ -632,15 +632,15 @@ cudaError_t pf_pass(const PrefillArgs& a, cudaStream_t st) {
   }
   const int tiles = (a.T + kPfTile - 1) / kPfTile, n_heads = a.batch * (PASS == 1 ? a.heads_q : a.heads_kv);
   const int items2 = (tiles + 1) / 2;
-  return 2ll * items2 * n_heads >= 3ll * kPfSlots ? pf_launch(two, pf_smem(2), a, items2, n_heads, st)
-                                                  : pf_launch(one, pf_smem(1), a, tiles, n_heads, st);
+  return 2ll * items2 * n_heads >= 3ll * num_sms ? pf_launch(two, pf_smem(2), a, items2, n_heads, num_sms, st)
+                                                  : pf_launch(one, pf_smem(1), a, tiles, n_heads, num_sms, st);
 }
 
 }  // namespace
 
-cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st) {
-  const cudaError_t e = pf_pass<1>(a, st);
-  return e != cudaSuccess ? e : pf_pass<2>(a, st);
+cudaError_t launch_prefill(const PrefillArgs& a, int num_sms, cudaStream_t st) {
+  const cudaError_t e = pf_pass<1>(a, num_sms, st);
+  return e != cudaSuccess ? e : pf_pass<2>(a, num_sms, st);
 }
 
 }  // namespace mikv

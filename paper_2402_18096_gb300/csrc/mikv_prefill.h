@@ -11,8 +11,6 @@ namespace mikv {
 
 // A tile: 128 tokens x 128 channels (bf16).
 constexpr int kPfTile = 128;
-// Resident CTAs of the prefill kernels (one per SM, 152 SMs).
-constexpr int kPfSlots = 152;
 
 struct PrefillArgs {
   CUtensorMap map_q;  // q_pre rows [B * Hq * T][128] bf16, box 64 channels x 128 rows, 128B swizzle
@@ -34,6 +32,6 @@ inline size_t prefill_workspace_bytes(int batch, int heads_q, int T) {
   return kWsHeader + (stats + 255) / 256 * 256;
 }
 
-cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st);
+cudaError_t launch_prefill(const PrefillArgs& a, int num_sms, cudaStream_t st);
 
 }  // namespace mikv

@@ -45,7 +45,7 @@ struct QPArgs {
 constexpr int kQpRowsPerWarp = 4;
 constexpr int kQpBlockRows = 4 * kQpRowsPerWarp;      // rows of a round (16 of K and of V each)
 constexpr int kQpRoundsMax = 16;
-constexpr int kQpBlocks = 2 * 152 * 4;                // fewer rounds per block until the grid has this many blocks
+constexpr int kQpBlocksPerSm = 2 * 4;                 // fewer rounds per block until the grid has this many per SM
 
 // Packs one row's codes: w[k] = code of channel 16 l8 + 2 k | code of channel 16 l8 + 2 k + 1 << 16. A word of the row
 // collects the same k from the lanes that share it, so the row's words are transposed through the warp's shared memory
@@ -503,7 +503,7 @@ __global__ void __launch_bounds__(128) balancer_kernel(const uint32_t* ws, int H
 
 cudaError_t launch_quantize_pack(const mikv_shape& s, const mikv_cache& c, const void* k_src,
                                  const void* v_src, const int32_t* src_tok, int n_src,
-                                 const int32_t* rows, int n_rows, int lo_start, cudaStream_t st) {
+                                 const int32_t* rows, int n_rows, int lo_start, int num_sms, cudaStream_t st) {
   if (n_rows == 0) return cudaSuccess;
   QPArgs a = {};
   a.dbg = debug_status_word();
@@ -523,7 +523,8 @@ cudaError_t launch_quantize_pack(const mikv_shape& s, const mikv_cache& c, const
   a.lo_start = lo_start;
   a.lo_cap = s.lo_cap;
   const long long all = (long long)((n_rows + kQpBlockRows - 1) / kQpBlockRows) * s.batch * s.heads_kv;  // rounds in all
-  a.rounds = (int)(all / kQpBlocks < 1 ? 1 : all / kQpBlocks < kQpRoundsMax ? all / kQpBlocks : kQpRoundsMax);
+  const long long rounds = all / ((long long)num_sms * kQpBlocksPerSm);
+  a.rounds = (int)(rounds < 1 ? 1 : rounds < kQpRoundsMax ? rounds : kQpRoundsMax);
   const int per_block = a.rounds * kQpBlockRows;
   const dim3 grid((n_rows + per_block - 1) / per_block, s.batch * s.heads_kv);
   switch (s.bits) {
