@@ -79,7 +79,10 @@ __host__ __device__ constexpr LoUnit lo_unit_layout_kch(int bits, int group) {
   return u;
 }
 
-// The largest unit (at most 8 blocks) that fits one stage.
+// The largest unit (at most 8 blocks) that fits one stage. (8-bit important codes: one block, 4352 bytes. Stages of
+// 9216 bytes hold two, which took the step of the Mistral-7B shape with an INT8 important set from 240.6 to 232.7 us, but
+// their softmax is updated once for both: the outputs move by 2e-4 to 1e-3 and, on four of ten shapes, away from the
+// 64-bit result.)
 __host__ __device__ constexpr LoUnit lo_unit_layout(int bits, int group) {
   int n = 8;
   while (n > 1 && lo_unit_layout_n(bits, group, n).total > kUnitBytes) --n;

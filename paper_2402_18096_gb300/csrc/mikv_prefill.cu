@@ -18,7 +18,7 @@
 //    of a tile (measured: 0, 4, 8 and 16 MMAs a tile took 446, 726, 993 and 1466 clocks), so one thread alone leaves the
 //    tensor cores idle half of the time; the other's MMAs fill its gap. (N = 256 keeps them full from one thread, 1025
 //    clocks for eight MMAs, but then two accumulators fill the tensor memory and all sixteen epilogue warps share
-//    each: 1086 against 1022 us for the whole call below.)
+//    each: 1086 against then 1022 us for the first call below.)
 //  - Four accumulators, which fill the tensor memory, so that MMAs run under the arithmetic, and one streamed tile for
 //    two fixed ones (MT = 2), which halves the traffic from L2 per score (the 128-row tiles drew 7.9 TB/s).
 //  - Four sets of four epilogue warps. With MT = 2 each has an accumulator of its own, each warp taking whole rows of
@@ -37,9 +37,10 @@
 //    32, Hkv 8, T 300: 22.8 / 24.8 / 22.7; B 1, H 32, T 512: 18.4 / 20.5 / 16.6; B 8, H 32, T 300: 35.0 / 37.2 / 33.1;
 //    B 2, H 40, T 777: 42.4 / 49.4 / 37.2.)
 //
-// Where the time goes now (128 x 128 tile and pass, clocks per SM): some 950 of the 512 that exponentials and MMAs each
-// need; MMAs with no arithmetic behind them 770, the arithmetic with no MMAs 790 (pass 1) and 930 (pass 2, whose
-// normalisers come from shared memory). B 8, H 32, T 4096: 1211 -> 965 us; B 1, Hq 32 / Hkv 8, T 32768: 8.59 -> 6.87
+// Where the time goes (128 x 128 tile and pass, clocks per SM): 957 (pass 1) and 1075 (pass 2) of the 512 that
+// exponentials and MMAs each need. In timing-only variants of the form before (1010 on average) MMAs with no arithmetic
+// behind them took 770, the arithmetic with no MMAs 790 (pass 1) and 930 (pass 2, whose normalisers come from shared
+// memory). B 8, H 32, T 4096: 1211 -> 965 us; B 1, Hq 32 / Hkv 8, T 32768: 8.59 -> 6.87
 // ms against one CTA per 128-token tile with 64-token streamed tiles, two per SM.
 //
 // The CTA's warps specialise: sixteen take the accumulator rows with tcgen05.ld and do the softmax
@@ -512,9 +513,9 @@ __device__ __forceinline__ float pf_join(float own, Part part) {
 
 // ------------------------------------------------------------------------------- pass 1: row statistics
 //
-// Per query row the softmax normaliser is accumulated against a reference r (log2 units): the exact maximum
-// of the row's first tile, raised only when a later tile's sum would leave the fp32 range (a logit more than
-// 64 above r, rare), so most tiles need no maximum at all. The pair (r, sum_t 2^(s_t - r)) defines the same
+// Per query row each thread accumulates its share of the softmax normaliser against a reference r (log2 units): the
+// exact maximum of the first 32 columns it reads, raised only when a later sum would leave the fp32 range (a logit more
+// than 64 above r, rare), so most columns need no maximum at all. The pair (r, sum_t 2^(s_t - r)) defines the same
 // normaliser as the true maximum; the kernel stores its log2, r + log2(sum), negated (pass 2 adds it).
 
 template <int MT>

@@ -5,8 +5,7 @@
 // group minima and maxima come from the lane's channels and butterfly shuffles, scale and zero are
 // rounded to fp16 outward so the stored grid covers the group's range, codes are round-half-even of the
 // IEEE fp32 quotient (x - beta) / alpha (the Eq. 1 helpers of mikv_quant_rows.cuh, shared with the
-// one-row quantizer of the step tail), and the packed words are assembled by a reduce-scatter over the
-// lanes that share them.
+// one-row quantizer of the step tail), and the packed words are joined from the lanes that share them.
 #include "mikv_device.cuh"
 #include "mikv_internal.h"
 #include "mikv_quant_rows.cuh"
@@ -33,13 +32,13 @@ struct QPArgs {
 // Bulk quantize/pack (Eq. 1): eight lanes per row and four rows per warp. Lane l8 = lane & 7 of a row owns
 // channels 16 l8 .. 16 l8 + 15 (two 16-byte loads), so a group's scale and zero are computed by GROUP / 16
 // lanes, and in the packed layout every channel of the lane sits at field index m = l8 of its 16-bit unit:
-// the lane's codes form partial words at fixed positions, which a reduce-scatter over the lanes that share
-// them turns into whole words, one or two per lane.
+// the lane's codes form partial words at fixed positions, joined with those of the lanes that share them into whole
+// words, one or two per lane (qp_store_codes).
 // It is bound by instruction issue (a row's bytes move in a third of the time its scalar arithmetic took), so the
 // arithmetic is packed: pairs of channels in fp32x2, minima and maxima three at a time, the code taken from the
 // rounded sum's low bits without a clamp, the doubtful codes found by one maximum over the lane's channels, the words
 // joined on the FMA pipe. A warp walks several rounds of rows with the next rows' loads in flight behind the
-// arithmetic; the balancer waits in shared memory, which leaves 60 registers and four blocks per SM (70 registers and
+// arithmetic; the balancer waits in shared memory, which leaves 61 registers and four blocks per SM (70 registers and
 // three blocks: 1230 us). B 32, Hkv 8, 26214 rows of K and V each, INT2 g32: 1839 -> 1086 us (the bytes at the copy
 // rate: 600).
 constexpr int kQpRowsPerWarp = 4;

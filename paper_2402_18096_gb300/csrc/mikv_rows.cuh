@@ -26,7 +26,8 @@ __device__ __forceinline__ int owner_warp(long long U, long long n_units, int n_
 // w + bh, each a normalised output with its (max, sum). merge_stats_warp gives every lane (M, L) = (max
 // logit, sum of exp(logit - M)); merge_output_warp gives lane l the output of channels 4l..4l+3, the
 // partials weighted by exp(max - M) * sum, over L. The per-slot statistics are read by all lanes at once
-// and broadcast with shuffles, so a merge costs a few dependent loads whatever the slot count.
+// and broadcast with shuffles; the outputs are read four partials at a time by the one warp, so a head of many
+// partials (228 for one request of 32768 tokens with 8 KV heads) takes a quarter as many rounds of loads in a row.
 __device__ __forceinline__ float merge_weight(const float* part_ml, int G, int bh, int jh, int w0, int i, float M) {
   constexpr float kLog2e = 1.4426950408889634f;
   const size_t slot = (size_t)(w0 + i + bh);
